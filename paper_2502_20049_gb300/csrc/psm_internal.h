@@ -239,6 +239,7 @@ struct IoParams {
   void* f;
   int layout;  // Layout
   double ghost[27];
+  float ghostf[27];  // the same in FP32 (a conversion in the kernel is an FP64 instruction per thread)
   double rho0;
   int z_begin, z_end;  // z-planes handled by this launch
   // import: from a natural FP64 state chunk (f_in, planes z_begin..z_end), uniform

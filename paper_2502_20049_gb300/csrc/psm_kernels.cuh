@@ -1595,115 +1595,239 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
 }
 
 // ---------------------------------------------------------------------------
-// Import / export / diagnostics (one thread per cell of planes [z_begin, z_end))
+// Import / export / diagnostics (one thread per cell of planes [z_begin, z_end)).
+// An FP64 instruction (conversions from and to double included) costs about
+// 64 FP32 ones on GB300, so a kernel with more than about 20 of them per cell
+// runs below the memory's rate: conversions between double and the narrower
+// types are integer operations on the bits (exact, the same values as the
+// conversion instructions), and k_macro sums in integers.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool io_cell(const IoParams& p, long long idx, int& x, int& y, int& z, long long& cell) {
-  const long long plane = (long long)p.g.nx * p.g.ny;
-  const long long n = plane * (p.z_end - p.z_begin);
-  if (idx >= n) return false;
-  z = p.z_begin + (int)(idx / plane);
-  const long long r = idx % plane;
-  y = (int)(r / p.g.nx);
-  x = (int)(r % p.g.nx);
-  cell = (long long)z * plane + r;
-  return true;
+__device__ __forceinline__ unsigned io_plane(const IoParams& p) { return (unsigned)p.g.nx * (unsigned)p.g.ny; }
+
+// The conversion instructions, for the values the bit operations leave out
+// (out of line: inline, the compiler would run them for every value and select).
+static __device__ __noinline__ double widen_rare(float f) { return (double)f; }
+template <class S>
+static __device__ __noinline__ S narrow_rare(double d) { return Store<S>::from_double(d); }
+
+// double(f): sign, exponent and mantissa moved to their places
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  if (m - 1u < 0x007fffffu || m >= 0x7f800000u) return widen_rare(f);  // subnormals, infinities, NaN
+  const unsigned hi = (b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// d rounded to the storage type (to nearest, ties to even) as one rounding.
+// In the float's normal range the float's bits are cut out of the double's:
+// for float storage rounded to nearest even, for 16-bit storage with the
+// discarded bits or-ed into the last one (24 bits rounded to odd, which rounds
+// on to 11 or 8 bits as the double itself would).
+template <class S>
+__device__ __forceinline__ S narrow(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), m = hi & 0x7fffffffu;
+  // exponents of [2^-126, 2^127): below the smallest normal float, or so large
+  // that rounding could overflow, the conversion instruction decides
+  if (m - 0x38100000u >= 0x0fd00000u) {
+    if ((m | lo) == 0u) return Store<S>::from_double(d);
+    return Store<S>::from_double(d);
+  }
+  const unsigned top = ((m - 0x38000000u) << 3) | (lo >> 29);
+  if constexpr (sizeof(S) == 4) {
+    const unsigned rest = lo << 3;  // the 29 discarded bits, left-justified
+    const unsigned up = (rest > 0x80000000u || (rest == 0x80000000u && (top & 1u))) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (top + up));
+  } else {
+    S r;
+    Store<S>::st(&r, __uint_as_float((hi & 0x80000000u) | top | ((lo << 3) ? 1u : 0u)));
+    return r;
+  }
+}
+template <>
+__device__ __forceinline__ double narrow<double>(double d) { return d; }
+
+template <class T>
+__device__ __forceinline__ T io_ghost(const IoParams& p, int i) {
+  if constexpr (sizeof(T) == 4) return p.ghostf[i];
+  else return p.ghost[i];
 }
 
 // f_i(x) (shifted) of a state stored in `layout`, ghost value for populations
 // entering from a ghost plane
 template <class S, int Q>
-__device__ __forceinline__ void read_state(const IoParams& p, const S* buf, const Nbr& nbr, long long cell,
-                                           typename Store<S>::T f[Q]) {
+__device__ __forceinline__ void read_state(const IoParams& p, const S* buf, unsigned cell,
+                                           typename Store<S>::T (&f)[Q]) {
   using T = typename Store<S>::T;
   const long long N = p.g.ncell;
+  const unsigned plane = io_plane(p);
+  if (p.layout == LAYOUT_SWAPPED) {
+    const unsigned z = cell / plane, r = cell - z * plane, y = r / (unsigned)p.g.nx;
+    Nbr nbr;
+    nbr.init(p.g, (int)(r - y * (unsigned)p.g.nx), (int)y, (int)z);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    if (nbr.from_ghost(lat_cz(i))) {
-      f[i] = T(p.ghost[i]);
-    } else if (p.layout == LAYOUT_SWAPPED) {
-      f[i] = Store<S>::ld(buf + (long long)lat_opp(i) * N +
-                          (unsigned)((unsigned)cell + nbr.off(-lat_cx(i), -lat_cy(i), -lat_cz(i))));
-    } else {
-      f[i] = Store<S>::ld(buf + (long long)i * N + cell);
+    for (int i = 0; i < Q; ++i) {
+      if (nbr.from_ghost(lat_cz(i))) f[i] = io_ghost<T>(p, i);
+      else
+        f[i] = Store<S>::ld(buf + (long long)lat_opp(i) * N +
+                            (unsigned)(cell + nbr.off(-lat_cx(i), -lat_cy(i), -lat_cz(i))));
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < Q; ++i) f[i] = Store<S>::ld(buf + (long long)i * N + cell);
+  if (p.g.bc_z == PSM_BC_EQ_INLET_OUTLET) {
+    const bool lo = cell < plane, hi = cell >= (unsigned)N - plane;
+    if (lo || hi) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+        if ((lat_cz(i) > 0 && lo) || (lat_cz(i) < 0 && hi)) f[i] = io_ghost<T>(p, i);
     }
   }
 }
 
+// f^eq_i(rho, u) - w_i rho0 in FP64 (initial states), separately rounded
+__device__ __forceinline__ double eq_shifted(double w, double cu, double rho, double uu, double rho0) {
+  const double e = __fma_rn(-1.5, uu, __fma_rn(__dmul_rn(4.5, cu), cu, __fma_rn(3.0, cu, 1.0)));
+  return __fma_rn(-w, rho0, __dmul_rn(__dmul_rn(w, rho), e));
+}
+__device__ __forceinline__ double uu64(const double* u) {
+  return __fma_rn(u[2], u[2], __fma_rn(u[1], u[1], __dmul_rn(u[0], u[0])));
+}
+__device__ __forceinline__ double cu64(int cx, int cy, int cz, const double* u) {
+  return __dadd_rn(__dadd_rn((double)cx * u[0], (double)cy * u[1]), (double)cz * u[2]);
+}
+
+// Uniform equilibrium: slot blockIdx.y of the stored layout filled with its
+// one value over the planes that are stored (populations entering from a ghost
+// plane are not), 16 bytes per store.  Bound by the write bandwidth; one value
+// per block instead of FP64 arithmetic per cell and direction took a 128^3
+// FP32 D3Q19 state (160 MB) from 1990 us to 39 us a call.
+constexpr unsigned FILL_BLOCK_BYTES = 65536;
 template <class S, int Q>
-__global__ void k_import(const __grid_constant__ IoParams p) {
+__global__ void __launch_bounds__(PSM_THREADS) k_fill_uniform(const __grid_constant__ IoParams p) {
+  const int slot = blockIdx.y;
+  // the population a slot holds; swapped: that of x + c_i, so the planes shift by c_z
+  const int i = p.layout == LAYOUT_SWAPPED ? lat_opp(slot) : slot;
+  const int cx = lat_c_rt(kLatCX, i), cy = lat_c_rt(kLatCY, i), cz = lat_c_rt(kLatCZ, i);
+  __shared__ S s_v;
+  if (threadIdx.x == 0) {
+    const int cls = cx * cx + cy * cy + cz * cz;
+    const double w = cls == 0 ? lat_w<Q>(0) : (cls == 1 ? lat_w<Q>(1) : (cls == 2 ? lat_w<Q>(7) : lat_w<Q>(Q - 1)));
+    s_v = Store<S>::from_double(eq_shifted(w, cu64(cx, cy, cz, p.u), p.rho, uu64(p.u), p.rho0));
+  }
+  __syncthreads();
+  const S v = s_v;
+  int z0 = 0, z1 = p.g.nz;
+  if (p.g.bc_z == PSM_BC_EQ_INLET_OUTLET && cz != 0) {
+    const bool drop_first = (cz > 0) != (p.layout == LAYOUT_SWAPPED);
+    if (drop_first) z0 = 1;
+    else z1 = p.g.nz - 1;
+  }
+  const unsigned long long plane = io_plane(p);
+  unsigned char* a = reinterpret_cast<unsigned char*>(static_cast<S*>(p.f) + (unsigned long long)slot * p.g.ncell + z0 * plane);
+  unsigned char* b = reinterpret_cast<unsigned char*>(static_cast<S*>(p.f) + (unsigned long long)slot * p.g.ncell + z1 * plane);
+  union {
+    uint4 q;
+    S e[16 / sizeof(S)];
+  } pk;
+#pragma unroll
+  for (int k = 0; k < (int)(16 / sizeof(S)); ++k) pk.e[k] = v;
+  // 16-byte pieces counted from the boundary below the range; the first and
+  // the last may hold values outside it
+  unsigned char* base = a - (reinterpret_cast<unsigned long long>(a) & 15ull);
+  for (unsigned long long blk = blockIdx.x;; blk += gridDim.x) {
+    unsigned char* c = base + blk * FILL_BLOCK_BYTES;
+    if (c >= b) return;
+#pragma unroll 4
+    for (unsigned o = threadIdx.x * 16u; o < FILL_BLOCK_BYTES; o += PSM_THREADS * 16u) {
+      unsigned char* q = c + o;
+      if (q >= a && q + 16 <= b) *reinterpret_cast<uint4*>(q) = pk.q;
+      else
+        for (int k = 0; k < (int)(16 / sizeof(S)); ++k)
+          if (q + k * sizeof(S) >= a && q + (k + 1) * sizeof(S) <= b) reinterpret_cast<S*>(q)[k] = v;
+    }
+  }
+}
+
+// A natural, unshifted FP64 state (or equilibria of per-cell fields, FIELD)
+// into the stored layout.  Bound by memory (8 Q bytes read, the storage type
+// written) with one FP64 operation per value: psm_set_state of a 256x256x192
+// FP32 state in device memory 496 us (2.9 GB), with the staging 6330 us.
+template <class S, int Q, bool FIELD>
+__global__ void __launch_bounds__(PSM_THREADS) k_import(const __grid_constant__ IoParams p) {
   S* buf = static_cast<S*>(p.f);
   const long long N = p.g.ncell;
-  const long long plane = (long long)p.g.nx * p.g.ny;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;; idx += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    long long cell;
-    if (!io_cell(p, idx, x, y, z, cell)) return;
-    Nbr nbr;
-    nbr.init(p.g, x, y, z);
-    for (int i = 0; i < Q; ++i) {
-      double v;
-      if (p.uniform || p.rho_f) {
-        const long long lc = cell - (long long)p.z_begin * plane;
-        const double* uc = p.rho_f ? p.u_f + 3 * lc : p.u;
-        const double rc = p.rho_f ? p.rho_f[lc] : p.rho;
-        const double cu = lat_cx(i) * uc[0] + lat_cy(i) * uc[1] + lat_cz(i) * uc[2];
-        const double uu = uc[0] * uc[0] + uc[1] * uc[1] + uc[2] * uc[2];
-        v = lat_w<Q>(i) * rc * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
-      } else {
-        v = p.f_in[(long long)i * plane * (p.z_end - p.z_begin) + (cell - (long long)p.z_begin * plane)];
-      }
-      v -= lat_w<Q>(i) * p.rho0;
-      if (nbr.from_ghost(lat_cz(i))) continue;  // such populations always read the ghost value
-      long long dstc;
-      int slot;
-      if (p.layout == LAYOUT_SWAPPED) {
-        slot = lat_opp(i);
-        dstc = (unsigned)((unsigned)cell + nbr.off(-lat_cx(i), -lat_cy(i), -lat_cz(i)));
-      } else {
-        slot = i;
-        dstc = cell;
-      }
-      buf[(long long)slot * N + dstc] = Store<S>::from_double(v);
+  const unsigned plane = io_plane(p);
+  const long long n = (long long)plane * (p.z_end - p.z_begin);
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const unsigned cell = (unsigned)p.z_begin * plane + (unsigned)idx;
+    double v[Q];
+    if constexpr (FIELD) {
+      const double u[3] = {p.u_f[3 * idx], p.u_f[3 * idx + 1], p.u_f[3 * idx + 2]};
+      const double rc = p.rho_f[idx], uu = uu64(u);
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+        v[i] = eq_shifted(lat_w<Q>(i), cu64(lat_cx(i), lat_cy(i), lat_cz(i), u), rc, uu, p.rho0);
+    } else {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) v[i] = __ldcs(p.f_in + (long long)i * n + idx);
+#pragma unroll
+      for (int i = 0; i < Q; ++i) v[i] = __fma_rn(-lat_w<Q>(i), p.rho0, v[i]);
+    }
+    const bool ghost = p.g.bc_z == PSM_BC_EQ_INLET_OUTLET;
+    const bool lo = ghost && cell < plane, hi = ghost && cell >= (unsigned)N - plane;
+    if (p.layout == LAYOUT_SWAPPED) {
+      const unsigned z = cell / plane, r = cell - z * plane, y = r / (unsigned)p.g.nx;
+      Nbr nbr;
+      nbr.init(p.g, (int)(r - y * (unsigned)p.g.nx), (int)y, (int)z);
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+        if (!nbr.from_ghost(lat_cz(i)))  // such populations always read the ghost value
+          buf[(long long)lat_opp(i) * N + (unsigned)(cell + nbr.off(-lat_cx(i), -lat_cy(i), -lat_cz(i)))] =
+              narrow<S>(v[i]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+        if (!((lat_cz(i) > 0 && lo) || (lat_cz(i) < 0 && hi))) buf[(long long)i * N + cell] = narrow<S>(v[i]);
     }
   }
 }
 
+// Natural, unshifted FP64.  Bound by memory (the storage type read, 8 Q bytes
+// written) with one FP64 operation per value: psm_get_state of a 256x256x192
+// FP32 state to device memory 503 us (2.9 GB), with the staging 4290 us.
 template <class S, int Q>
-__global__ void k_export(const __grid_constant__ IoParams p) {
+__global__ void __launch_bounds__(PSM_THREADS) k_export(const __grid_constant__ IoParams p) {
   using T = typename Store<S>::T;
   const S* buf = static_cast<const S*>(p.f);
-  const long long plane = (long long)p.g.nx * p.g.ny;
-  const long long nchunk = plane * (p.z_end - p.z_begin);
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;; idx += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    long long cell;
-    if (!io_cell(p, idx, x, y, z, cell)) return;
-    Nbr nbr;
-    nbr.init(p.g, x, y, z);
+  const unsigned plane = io_plane(p);
+  const long long n = (long long)plane * (p.z_end - p.z_begin);
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
+       idx += (long long)gridDim.x * blockDim.x) {
     T f[Q];
-    read_state<S, Q>(p, buf, nbr, cell, f);
-    for (int i = 0; i < Q; ++i) p.f_out[(long long)i * nchunk + idx] = (double)f[i] + lat_w<Q>(i) * p.rho0;
+    read_state<S, Q>(p, buf, (unsigned)p.z_begin * plane + (unsigned)idx, f);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) __stcs(p.f_out + (long long)i * n + idx, __fma_rn(lat_w<Q>(i), p.rho0, widen(f[i])));
   }
 }
 
 // Natural layout, shifted, storage precision (psm_get_pdfs): the stored
 // values themselves (ghost-plane populations as the ghost value, rounded).
 template <class S, int Q>
-__global__ void k_export_raw(const __grid_constant__ IoParams p) {
+__global__ void __launch_bounds__(PSM_THREADS) k_export_raw(const __grid_constant__ IoParams p) {
   using T = typename Store<S>::T;
   const S* buf = static_cast<const S*>(p.f);
   S* out = static_cast<S*>(p.f_out_raw);
-  const long long plane = (long long)p.g.nx * p.g.ny;
-  const long long nchunk = plane * (p.z_end - p.z_begin);
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;; idx += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    long long cell;
-    if (!io_cell(p, idx, x, y, z, cell)) return;
-    Nbr nbr;
-    nbr.init(p.g, x, y, z);
+  const unsigned plane = io_plane(p);
+  const long long n = (long long)plane * (p.z_end - p.z_begin);
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
+       idx += (long long)gridDim.x * blockDim.x) {
     T f[Q];
-    read_state<S, Q>(p, buf, nbr, cell, f);
-    for (int i = 0; i < Q; ++i) Store<S>::st(out + (long long)i * nchunk + idx, f[i]);
+    read_state<S, Q>(p, buf, (unsigned)p.z_begin * plane + (unsigned)idx, f);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) Store<S>::st(out + (long long)i * n + idx, f[i]);
   }
 }
 
@@ -1712,44 +1836,151 @@ template <class S, int Q>
 __global__ void k_get_cells(const __grid_constant__ IoParams p, const long long* cells, long long n, double* out) {
   using T = typename Store<S>::T;
   const S* buf = static_cast<const S*>(p.f);
-  const long long plane = (long long)p.g.nx * p.g.ny;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
     const long long cell = cells[k];
     if (cell < 0 || cell >= p.g.ncell) continue;  // the host validates; never read out of bounds
-    const int z = (int)(cell / plane);
-    const long long r = cell % plane;
-    const int y = (int)(r / p.g.nx), x = (int)(r % p.g.nx);
-    Nbr nbr;
-    nbr.init(p.g, x, y, z);
     T f[Q];
-    read_state<S, Q>(p, buf, nbr, cell, f);
+    read_state<S, Q>(p, buf, (unsigned)cell, f);
     for (int i = 0; i < Q; ++i) out[k * Q + i] = (double)f[i] + lat_w<Q>(i) * p.rho0;
   }
 }
 
+// Density and velocity with FP64 sums and divisions.
+template <class T, int Q>
+__device__ __forceinline__ void macro64(const T* f, double rho0, double& rho, double* u) {
+  double drho = 0, j[3] = {0, 0, 0};
+  for (int i = 0; i < Q; ++i) {
+    const double v = (double)f[i];
+    drho += v;
+    j[0] += lat_cx(i) * v;
+    j[1] += lat_cy(i) * v;
+    j[2] += lat_cz(i) * v;
+  }
+  rho = rho0 + drho;
+  for (int k = 0; k < 3; ++k) u[k] = j[k] / rho;
+}
+
+template <int Q>
+static __device__ __noinline__ void macro64_rare(const float* f, double rho0, double* out) {
+  macro64<float, Q>(f, rho0, out[0], out + 1);
+}
+static __device__ __noinline__ double add_tail(double x, int n) { return __fma_rn((double)n, 1.1920928955078125e-07, x); }
+
+// The same from float populations with the sums in integers: 16 FP64
+// operations per cell instead of about 100.  The populations are scaled by a
+// power of two (exactly) so that the largest lies in [1, 2), and each is cut
+// into three integers, multiples of 2^-21, 2^-44 and 2^-67, by adding 1.5 times
+// the power of two whose last place that is (the sum's bits then count from the
+// constant's): no value loses a bit above 2^-68 of the largest, and integer
+// sums are exact, so drho and j are their exact values rounded once (FP64 sums
+// round after every term at 2^-53).  u = j / rho: a reciprocal from
+// rcp.approx with one Newton step, then the quotient corrected by its own
+// remainder, rounded as the division is but for ties in the 2^-27 tail.
+// false (nothing written) for populations or densities outside the range the
+// cuts are made for (also infinities and NaN): macro64 decides those.
+template <int Q>
+__device__ __forceinline__ bool macro_int(const float (&f)[Q], double rho0, double& rho, double (&u)[3]) {
+  unsigned big = 0u;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) big = max(big, __float_as_uint(f[i]) & 0x7fffffffu);
+  const int E = (int)(big >> 23);
+  if (E < 30 || E > 250) {
+    if (big != 0u) return false;
+    rho = rho0;
+    u[0] = u[1] = u[2] = 0.0;
+    return rho0 > 0.0;
+  }
+  const float scale = __uint_as_float((unsigned)(254 - E) << 23);  // 2^(127 - E)
+  const float M1 = 6.0f, M2 = 7.152557373046875e-07f, M3 = 8.526512829121202e-14f;  // 1.5 2^2, 2^-21, 2^-44
+  int n1[4] = {0, 0, 0, 0}, n2[4] = {0, 0, 0, 0}, n3[4] = {0, 0, 0, 0};  // sums: 1, c_x, c_y, c_z
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const float g = __fmul_rn(f[i], scale);
+    const float t1 = __fadd_rn(g, M1), r1 = __fsub_rn(g, __fsub_rn(t1, M1));
+    const float t2 = __fadd_rn(r1, M2), r2 = __fsub_rn(r1, __fsub_rn(t2, M2));
+    const float t3 = __fadd_rn(r2, M3);
+    const int a = __float_as_int(t1), b = __float_as_int(t2), c = __float_as_int(t3);
+    const int s[4] = {1, lat_cx(i), lat_cy(i), lat_cz(i)};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (s[k] > 0) n1[k] = (int)((unsigned)n1[k] + (unsigned)a), n2[k] = (int)((unsigned)n2[k] + (unsigned)b), n3[k] = (int)((unsigned)n3[k] + (unsigned)c);
+      if (s[k] < 0) n1[k] = (int)((unsigned)n1[k] - (unsigned)a), n2[k] = (int)((unsigned)n2[k] - (unsigned)b), n3[k] = (int)((unsigned)n3[k] - (unsigned)c);
+    }
+  }
+  // the constants' own bits cancel in the sums over c (as many +1 as -1)
+  n1[0] = (int)((unsigned)n1[0] - (unsigned)Q * __float_as_uint(M1));
+  n2[0] = (int)((unsigned)n2[0] - (unsigned)Q * __float_as_uint(M2));
+  n3[0] = (int)((unsigned)n3[0] - (unsigned)Q * __float_as_uint(M3));
+  double X[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    // (n1 2^23 + n2) as a double, exactly: below 2^51 in size
+    const long long v = (long long)n1[k] * (1ll << 23) + (long long)n2[k];
+    X[k] = __dsub_rn(__longlong_as_double(0x4338000000000000ll + v), 6755399441055744.0);
+  }
+  if (n3[0] | n3[1] | n3[2] | n3[3]) {  // values below 2^-20 of the largest: n3 2^-23 more
+#pragma unroll
+    for (int k = 0; k < 4; ++k) X[k] = add_tail(X[k], n3[k]);
+  }
+  const int sh = E - 171;  // X counts in units of 2^(E - 127 - 44)
+  const double rh = __fma_rn(X[0], __hiloint2double((1023 + sh) << 20, 0), rho0);
+  const unsigned rb = (unsigned)__double2hiint(rh);
+  if (rb - (923u << 20) >= (200u << 20)) return false;  // not in [2^-100, 2^100)
+  rho = rh;
+  float a;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(__uint_as_float((rb - 0x38000000u) << 3)));
+  const unsigned ab = __float_as_uint(a);
+  const double inv0 = __hiloint2double((int)((ab >> 3) + 0x38000000u), (int)(ab << 29));
+  const double inv = __fma_rn(inv0, __fma_rn(-rh, inv0, 1.0), inv0);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double q0 = __dmul_rn(X[k + 1], inv);
+    const double q = __fma_rn(__fma_rn(-q0, rh, X[k + 1]), inv, q0);
+    const int qh = __double2hiint(q), ql = __double2loint(q);
+    // q 2^sh: |q| is 0 or lies in [2^-124, 2^151], so the exponent field stays in range
+    u[k] = ((qh & 0x7fffffff) | ql) ? __hiloint2double(qh + (sh << 20), ql) : 0.0;
+  }
+  return true;
+}
+
+// Density and velocity (psm_get_macroscopic).  The velocities of a warp's
+// cells pass through shared memory so that the stores are contiguous.  Bound by
+// the FP64 pipe (16 instructions per cell): a 256x256x192 FP32 state to device
+// memory in 403 us (1.4 GB; FP64 sums and divisions and a staging chunk: 3290 us).
 template <class S, int Q>
-__global__ void k_macro(const __grid_constant__ IoParams p) {
+__global__ void __launch_bounds__(PSM_THREADS) k_macro(const __grid_constant__ IoParams p) {
   using T = typename Store<S>::T;
   const S* buf = static_cast<const S*>(p.f);
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;; idx += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    long long cell;
-    if (!io_cell(p, idx, x, y, z, cell)) return;
-    Nbr nbr;
-    nbr.init(p.g, x, y, z);
-    T f[Q];
-    read_state<S, Q>(p, buf, nbr, cell, f);
-    double drho = 0, j[3] = {0, 0, 0};
-    for (int i = 0; i < Q; ++i) {
-      const double v = (double)f[i];
-      drho += v;
-      j[0] += lat_cx(i) * v;
-      j[1] += lat_cy(i) * v;
-      j[2] += lat_cz(i) * v;
+  __shared__ double s_u[PSM_THREADS / 32][96];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned plane = io_plane(p);
+  const long long n = (long long)plane * (p.z_end - p.z_begin);
+  for (long long w0 = blockIdx.x * (long long)blockDim.x + warp * 32; w0 < n; w0 += (long long)gridDim.x * blockDim.x) {
+    const long long idx = w0 + lane;
+    if (idx < n) {
+      T f[Q];
+      read_state<S, Q>(p, buf, (unsigned)p.z_begin * plane + (unsigned)idx, f);
+      double rho, u[3];
+      if constexpr (sizeof(T) == 4) {
+        if (!macro_int<Q>(f, p.rho0, rho, u)) {
+          float g[Q];
+          double r[4];
+#pragma unroll
+          for (int i = 0; i < Q; ++i) g[i] = f[i];
+          macro64_rare<Q>(g, p.rho0, r);
+          rho = r[0], u[0] = r[1], u[1] = r[2], u[2] = r[3];
+        }
+      } else {
+        macro64<T, Q>(f, p.rho0, rho, u);
+      }
+      __stcs(p.rho_out + idx, rho);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) s_u[warp][3 * lane + k] = u[k];
     }
-    const double rho = p.rho0 + drho;
-    p.rho_out[idx] = rho;
-    for (int k = 0; k < 3; ++k) p.u_out[3 * idx + k] = j[k] / rho;
+    __syncwarp();
+    const int m = (int)(n - w0 < 32 ? n - w0 : 32) * 3;
+    for (int k = lane; k < m; k += 32) __stcs(p.u_out + 3 * w0 + k, s_u[warp][k]);
+    __syncwarp();
   }
 }
 
@@ -1758,14 +1989,12 @@ __global__ void __launch_bounds__(PSM_THREADS) k_mass(const __grid_constant__ Io
   using T = typename Store<S>::T;
   const S* buf = static_cast<const S*>(p.f);
   double acc = 0.0;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;; idx += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    long long cell;
-    if (!io_cell(p, idx, x, y, z, cell)) break;
-    Nbr nbr;
-    nbr.init(p.g, x, y, z);
+  const unsigned plane = io_plane(p);
+  const long long n = (long long)plane * (p.z_end - p.z_begin);
+  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
+       idx += (long long)gridDim.x * blockDim.x) {
     T f[Q];
-    read_state<S, Q>(p, buf, nbr, cell, f);
+    read_state<S, Q>(p, buf, (unsigned)p.z_begin * plane + (unsigned)idx, f);
     double m = p.rho0;
     for (int i = 0; i < Q; ++i) m += (double)f[i];
     acc += m;
@@ -1909,8 +2138,23 @@ cudaError_t launch_step_q(int mode, int fl, const StepParams& p, cudaStream_t st
 inline long long io_cells(const IoParams& p) { return (long long)p.g.nx * p.g.ny * (p.z_end - p.z_begin); }
 inline int io_grid(const IoParams& p) {
   long long b = (io_cells(p) + PSM_THREADS - 1) / PSM_THREADS;
-  if (b > 4096) b = 4096;
+  if (b > (1 << 20)) b = 1 << 20;
   return (int)(b < 1 ? 1 : b);
+}
+
+template <class S, int Q>
+cudaError_t launch_import_q(const IoParams& p, cudaStream_t st) {
+  if (p.uniform) {
+    const unsigned long long bytes = (unsigned long long)p.g.ncell * sizeof(S) + 16;
+    unsigned long long b = (bytes + FILL_BLOCK_BYTES - 1) / FILL_BLOCK_BYTES;
+    if (b > (1u << 20)) b = 1u << 20;
+    k_fill_uniform<S, Q><<<dim3((unsigned)b, Q), PSM_THREADS, 0, st>>>(p);
+  } else if (p.rho_f) {
+    k_import<S, Q, true><<<io_grid(p), PSM_THREADS, 0, st>>>(p);
+  } else {
+    k_import<S, Q, false><<<io_grid(p), PSM_THREADS, 0, st>>>(p);
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace psm
@@ -1933,9 +2177,7 @@ inline int io_grid(const IoParams& p) {
     else tma_layout_q<S, 27>(mode, fl, out);                                                            \
   }                                                                                                     \
   cudaError_t launch_import_##NAME(int Q, const IoParams& p, cudaStream_t st) {                         \
-    if (Q == 19) k_import<S, 19><<<io_grid(p), PSM_THREADS, 0, st>>>(p);                                \
-    else k_import<S, 27><<<io_grid(p), PSM_THREADS, 0, st>>>(p);                                        \
-    return cudaGetLastError();                                                                          \
+    return Q == 19 ? launch_import_q<S, 19>(p, st) : launch_import_q<S, 27>(p, st);                     \
   }                                                                                                     \
   cudaError_t launch_export_##NAME(int Q, const IoParams& p, cudaStream_t st) {                         \
     if (Q == 19) k_export<S, 19><<<io_grid(p), PSM_THREADS, 0, st>>>(p);                                \
