@@ -367,90 +367,6 @@ cudaError_t launch_occupancy(const unsigned long long* bricks, int gx, int gy, i
   return cudaGetLastError();
 }
 
-// One semi-implicit Euler step of the rigid-body equations per body in mask
-// (thread b), from this step's force and torque on the body ft[b][6]:
-//   v += (F + Fext) / m,  R += v,  L += T + Text,
-//   Q <- Rot(w*) Q, w* = Q Ib^-1 Q^T L,  w = Q Ib^-1 Q^T L,
-// then the DevBody of the next step (kinematics, the cell box of the rotated
-// geometry box widened by 2.5 cells, the remap's pose and its float form).
-__device__ void q_ibinv_qt(const double* Q, const double* Ibinv, const double* L, double* w) {
-  double a[3], b[3];
-  for (int i = 0; i < 3; ++i) a[i] = Q[i] * L[0] + Q[3 + i] * L[1] + Q[6 + i] * L[2];
-  for (int i = 0; i < 3; ++i) b[i] = Ibinv[3 * i] * a[0] + Ibinv[3 * i + 1] * a[1] + Ibinv[3 * i + 2] * a[2];
-  for (int i = 0; i < 3; ++i) w[i] = Q[3 * i] * b[0] + Q[3 * i + 1] * b[1] + Q[3 * i + 2] * b[2];
-}
-
-__global__ void k_body_update(BodyDyn* dyn, DevBody* dev, const double* ft, unsigned mask, int nb, int nx, int ny,
-                              int nz) {
-  const int b = threadIdx.x;
-  if (b >= nb || !((mask >> b) & 1u)) return;
-  BodyDyn& S = dyn[b];
-  const double* F = ft + 6 * b;
-  for (int k = 0; k < 3; ++k) S.v[k] += (F[k] + S.Fext[k]) / S.mass;
-  for (int k = 0; k < 3; ++k) S.R[k] += S.v[k];
-  for (int k = 0; k < 3; ++k) S.L[k] += F[3 + k] + S.Text[k];
-  double ws[3];
-  q_ibinv_qt(S.Q, S.Ibinv, S.L, ws);
-  const double a = sqrt(ws[0] * ws[0] + ws[1] * ws[1] + ws[2] * ws[2]);
-  if (a > 0.0) {
-    const double k0 = ws[0] / a, k1 = ws[1] / a, k2 = ws[2] / a;
-    double sn, cs;
-    sincos(a, &sn, &cs);
-    const double oc = 1.0 - cs;
-    const double Rm[9] = {cs + oc * k0 * k0,      oc * k0 * k1 - sn * k2, oc * k0 * k2 + sn * k1,
-                          oc * k1 * k0 + sn * k2, cs + oc * k1 * k1,      oc * k1 * k2 - sn * k0,
-                          oc * k2 * k0 - sn * k1, oc * k2 * k1 + sn * k0, cs + oc * k2 * k2};
-    double Qn[9];
-    for (int r = 0; r < 3; ++r)
-      for (int c = 0; c < 3; ++c) Qn[3 * r + c] = Rm[3 * r] * S.Q[c] + Rm[3 * r + 1] * S.Q[3 + c] + Rm[3 * r + 2] * S.Q[6 + c];
-    for (int k = 0; k < 9; ++k) S.Q[k] = Qn[k];
-  }
-  q_ibinv_qt(S.Q, S.Ibinv, S.L, S.w);
-  DevBody& d = dev[b];
-  for (int k = 0; k < 3; ++k) {
-    d.Rf[k] = (float)S.R[k];
-    d.R[k] = S.R[k];
-    d.omega[k] = S.w[k];
-    d.v[k] = S.v[k];
-    d.omegaf[k] = (float)S.w[k];
-    d.vf[k] = (float)S.v[k];
-  }
-  double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-  const double ext[3] = {(double)S.gx, (double)S.gy, (double)S.gz};
-  for (int c = 0; c < 8; ++c) {
-    double pb[3];
-    for (int k = 0; k < 3; ++k) pb[k] = S.lo[k] + (((c >> k) & 1) ? ext[k] : 0.0);
-    for (int r = 0; r < 3; ++r) {
-      const double w = S.Q[3 * r] * pb[0] + S.Q[3 * r + 1] * pb[1] + S.Q[3 * r + 2] * pb[2] + S.R[r];
-      mn[r] = fmin(mn[r], w);
-      mx[r] = fmax(mx[r], w);
-    }
-  }
-  const int dims[3] = {nx, ny, nz};
-  int lo_[3], hi_[3];
-  for (int k = 0; k < 3; ++k) {
-    double a0 = floor(mn[k] - 2.5), e = ceil(mx[k] + 2.5) + 1.0;
-    if (a0 < 0) a0 = 0;
-    if (e > (double)dims[k]) e = (double)dims[k];
-    if (e < a0) e = a0;
-    lo_[k] = (int)a0;
-    hi_[k] = (int)e;
-  }
-  d.x0 = lo_[0];
-  d.x1 = hi_[0];
-  d.y0 = lo_[1];
-  d.y1 = hi_[1];
-  d.z0 = lo_[2];
-  d.z1 = hi_[2];
-  remap_setup(d, S.Q, S.R, S.lo);
-}
-
-cudaError_t launch_body_update(BodyDyn* dyn, DevBody* dev, const double* ft, unsigned mask, int nb, int nx, int ny,
-                               int nz, cudaStream_t st) {
-  k_body_update<<<1, 32, 0, st>>>(dyn, dev, ft, mask, nb, nx, ny, nz);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_remap(const RemapParams& p, cudaStream_t st) {
   long long cells = (long long)p.g.nx * p.g.ny * (p.z_end - p.z_begin);
   long long b = (cells + PSM_THREADS - 1) / PSM_THREADS;
@@ -1374,6 +1290,7 @@ int psm_step(psm_handle h, int n) {
     psm::set_slots(p, h->lat.storage, h->Q);
     p.free_mask = h->free_mask;
     p.dbody = h->d_dev_bodies;
+    p.dyn = h->d_dyn;
     // the AA odd step runs with plain loads unless its TMA variant applies
     const bool tma_now = use_tma && (mode != psm::MODE_AA_ODD ||
                                      (h->tma_odd_ok && (h->variant == PSM_KERNEL_TMA || !PSM_AA_ODD_PLAIN)));
@@ -1388,11 +1305,6 @@ int psm_step(psm_handle h, int n) {
     cudaError_t e = tma_now ? psm::launch_step_tma(h->lat.storage, h->Q, mode, p, tm, h->stream)
                             : psm::launch_step(h->lat.storage, h->Q, mode, p, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
-    if (h->free_mask) {
-      e = psm::launch_body_update(h->d_dyn, h->d_dev_bodies, p.ft_out, h->free_mask, h->nbodies, (int)h->grid.nx,
-                                  (int)h->grid.ny, (int)h->grid.nz, h->stream);
-      if (e != cudaSuccess) return cuda_fail(e, "body update launch");
-    }
     if (h->lat.streaming == PSM_STREAM_TWO_GRID) h->cur ^= 1;
     h->step++;
   }

@@ -213,7 +213,8 @@ struct StepParams {
   // bodies whose motion the device integrates (two-way coupling): bit b set ->
   // body b of this step is dbody[b] (device memory), not body[b]
   unsigned free_mask;
-  const DevBody* dbody;
+  DevBody* dbody;
+  BodyDyn* dyn;  // their state, advanced by the block that sums the loads
   const float* delta;  // optional additive eps perturbation per cell (nullptr: none)
   // force/torque reduction
   double* partials;      // [gridDim.x][nbodies * 6]
@@ -296,10 +297,6 @@ cudaError_t launch_export_raw(int storage, int Q, const IoParams& p, cudaStream_
 cudaError_t launch_macro(int storage, int Q, const IoParams& p, cudaStream_t st);
 cudaError_t launch_mass(int storage, int Q, const IoParams& p, int blocks, cudaStream_t st);
 cudaError_t launch_remap(const RemapParams& p, cudaStream_t st);
-// one rigid-body step of the bodies in `mask` from the force/torque series
-// entry ft (this step's) -> their DevBody of the next step
-cudaError_t launch_body_update(BodyDyn* dyn, DevBody* dev, const double* ft, unsigned mask, int nb, int nx, int ny,
-                               int nz, cudaStream_t st);
 // occupancy of a geometry field (DevBody::occ) from its bricks (device)
 cudaError_t launch_occupancy(const unsigned long long* bricks, int gx, int gy, int gz, int wpb, unsigned char* occ,
                              cudaStream_t st);

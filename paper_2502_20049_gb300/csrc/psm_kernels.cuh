@@ -1000,6 +1000,124 @@ __device__ __forceinline__ void psm_load(const StepParams& p, const Stencil& sn,
   }
 }
 
+// One semi-implicit Euler step of a free body's rigid-body equations (two-way
+// coupling) by one warp, from this step's force and torque on the body ft:
+//   v += (F + Fext) / m,  R += v,  L += T + Text,
+//   Q <- Rot(w*) Q, w* = Q Ib^-1 Q^T L,  w = Q Ib^-1 Q^T L,
+// then the DevBody of the next step (kinematics, the cell box of the rotated
+// geometry box widened by 2.5 cells, the remap's pose and its float form,
+// remap_setup).  Run by the block that summed the loads: a chain of FP64
+// operations that nothing overlaps, so the components and matrix elements go to
+// the lanes (one thread in a kernel of its own: 25 us a step; here about 7 us).
+static __device__ __noinline__ void body_update(BodyDyn* S, DevBody* d, const double* ft, int nx, int ny, int nz) {
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int k = lane % 3, r = (lane / 3) % 3;  // a vector's component; a matrix element (r, k) in lanes 0 .. 8
+  auto get = [&](double v, int src) { return __shfl_sync(all, v, src); };
+  auto sum3 = [](double a, double x, double b, double y, double c, double z) { return fma(a, x, fma(b, y, c * z)); };
+  const double v = S->v[k] + (ft[k] + S->Fext[k]) / S->mass;
+  const double R = S->R[k] + v;
+  const double L = S->L[k] + (ft[3 + k] + S->Text[k]);
+  double Q = S->Q[3 * r + k];
+  const double I0 = S->Ibinv[3 * k], I1 = S->Ibinv[3 * k + 1], I2 = S->Ibinv[3 * k + 2];
+  const double L0 = get(L, 0), L1 = get(L, 1), L2 = get(L, 2);
+  // component k of Q Ib^-1 Q^T L in every lane
+  auto spin = [&](double q) {
+    const double a = sum3(get(q, k), L0, get(q, 3 + k), L1, get(q, 6 + k), L2);
+    const double b = sum3(I0, get(a, 0), I1, get(a, 1), I2, get(a, 2));
+    return sum3(get(q, 3 * k), get(b, 0), get(q, 3 * k + 1), get(b, 1), get(q, 3 * k + 2), get(b, 2));
+  };
+  const double ws = spin(Q);
+  const double w0 = get(ws, 0), w1 = get(ws, 1), w2 = get(ws, 2);
+  const double a = sqrt(sum3(w0, w0, w1, w1, w2, w2));
+  if (a > 0.0) {  // the same in every lane
+    const double n = ws / a;
+    const double n0 = get(n, 0), n1 = get(n, 1), n2 = get(n, 2);
+    double sn, cs;
+    sincos(a, &sn, &cs);
+    const double nr = r == 0 ? n0 : (r == 1 ? n1 : n2), nk = k == 0 ? n0 : (k == 1 ? n1 : n2);
+    // Rodrigues: element (r, k) = cos d_rk + (1 - cos) n_r n_k + sin [n]x_rk
+    const int o = 3 - r - k;  // the third axis where r != k
+    const double no = o == 0 ? n0 : (o == 1 ? n1 : n2);
+    const double sgn = (k == (r + 1) % 3) ? -sn : sn;
+    const double Rm = r == k ? fma((1.0 - cs) * nr, nk, cs) : fma((1.0 - cs) * nr, nk, sgn * no);
+    Q = sum3(get(Rm, 3 * r), get(Q, k), get(Rm, 3 * r + 1), get(Q, 3 + k), get(Rm, 3 * r + 2), get(Q, 6 + k));
+  }
+  const double w = spin(Q);
+  if (lane < 3) {
+    S->v[k] = v, S->R[k] = R, S->L[k] = L, S->w[k] = w;
+    d->R[k] = R, d->v[k] = v, d->omega[k] = w;
+    d->Rf[k] = (float)R, d->vf[k] = (float)v, d->omegaf[k] = (float)w;
+  }
+  if (lane < 9) {
+    S->Q[lane] = Q;
+    d->Qd[lane] = Q;
+  }
+  // hull of the rotated geometry box: corner c, component k (lanes 3 c + k and, for corners 8 .. 10, copies)
+  const int c = (lane / 3) & 7;
+  const double lo0 = S->lo[0], lo1 = S->lo[1], lo2 = S->lo[2];
+  const double p0 = lo0 + ((c & 1) ? (double)S->gx : 0.0), p1 = lo1 + ((c & 2) ? (double)S->gy : 0.0),
+               p2 = lo2 + ((c & 4) ? (double)S->gz : 0.0);
+  const double wc = sum3(get(Q, 3 * k), p0, get(Q, 3 * k + 1), p1, get(Q, 3 * k + 2), p2) + R;
+  double mn = wc, mx = wc;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) {
+    const double t = get(wc, (3 * q + lane) % 24);  // lanes 0 .. 23 hold the eight corners
+    mn = fmin(mn, t);
+    mx = fmax(mx, t);
+  }
+  // (lanes 24 .. 31 repeat lanes 0 .. 7)
+  const int dim = k == 0 ? nx : (k == 1 ? ny : nz);
+  double b0d = floor(mn - 2.5), b1d = ceil(mx + 2.5) + 1.0;
+  if (b0d < 0.0) b0d = 0.0;
+  if (b1d > (double)dim) b1d = (double)dim;
+  if (b1d < b0d) b1d = b0d;
+  const int b0 = (int)b0d, b1 = (int)b1d;
+  if (lane < 3) {
+    int* lo_ = k == 0 ? &d->x0 : (k == 1 ? &d->y0 : &d->z0);
+    int* hi_ = k == 0 ? &d->x1 : (k == 1 ? &d->y1 : &d->z1);
+    *lo_ = b0;
+    *hi_ = b1;
+  }
+  // remap_setup with its components in the lanes
+  const double n = (double)(1 << d->s);
+  const double U = 5.9604644775390625e-08, Ud = 1.1102230246251565e-16;  // 2^-24, 2^-53
+  const int last = b1 > b0 ? b1 - 1 : b0;
+  const int anc = b0 + (last - b0) / 2;
+  const double be = fmax(fabs((double)(b0 - anc)), fabs((double)(last - anc)));
+  const double bd = fmax(fabs((double)b0 + 0.5 - R), fabs((double)last + 0.5 - R));
+  const double lok = k == 0 ? lo0 : (k == 1 ? lo1 : lo2);
+  const double Be = get(be, 0) + get(be, 1) + get(be, 2), Bd = get(bd, 0) + get(bd, 1) + get(bd, 2);
+  const double lom = fmax(fabs(lo0), fmax(fabs(lo1), fabs(lo2)));
+  const double ac = ((double)anc + 0.5) - R;
+  const double X = sum3(get(Q, k), get(ac, 0), get(Q, 3 + k), get(ac, 1), get(Q, 6 + k), get(ac, 2));
+  const double H = ((X - 0.5) - lok) * n + 0.5;
+  const double Hmax = fmax(fabs(get(H, 0)), fmax(fabs(get(H, 1)), fabs(get(H, 2))));
+  const double span = (Hmax + 1.0) + (n + 1.0) * Be;
+  // the finest grid 2^-m, m <= 20, on which the high parts stay below 2^24 (every m below it does too)
+  const unsigned fits = __ballot_sync(all, lane <= 20 && span * (double)(1 << min(lane, 20)) < 16777216.0);
+  const bool form = fits != 0u && span < 1e30;
+  const int m = form ? 31 - __clz(fits) : 0;
+  const double sc = (double)(1 << m), isc = 1.0 / sc;
+  const double G = Q * n, gh = floor(G * sc + 0.5) * isc, hh = floor(H * sc + 0.5) * isc;
+  if (lane < 9) {
+    d->Ghi[lane] = form ? (float)gh : 0.0f;
+    d->Glo[lane] = form ? (float)(G - gh) : 0.0f;
+  }
+  if (lane < 3) {
+    d->anchor[k] = anc;
+    d->lod[k] = lok;
+    d->Hhi[k] = form ? (float)hh : 0.0f;
+    d->Hlo[k] = form ? (float)(H - hh) : 0.0f;
+  }
+  if (lane == 0) {
+    const double Lb = 0.5 * isc * (1.0 + Be);
+    const double ef = U * 0.5 * isc * (1.0 + Be) + 3.0 * U * Lb + U * (1.0 + Lb);
+    const double ed = n * Ud * (7.0 * Bd + 3.0 * lom + 2.0) + Ud;
+    d->rtol = form ? (float)(2.0 * (ef + 2.0 * ed) + U) : 2.0f;
+  }
+}
+
 // Per-warp force/torque accumulation into s_ft[warp] (fixed order: warp
 // butterfly in the contribution's precision, then added in FP64 in tile
 // order).  All 32 lanes must call it.
@@ -1019,9 +1137,11 @@ __device__ __forceinline__ void warp_ft(double (*s_ft)[PSM_MAX_BODIES * 6], int 
   }
 }
 
-// Block sum of the per-warp slots (fixed order), then the grid-wide ordered sum.
+// Block sum of the per-warp slots (fixed order), then the grid-wide ordered
+// sum, and in the block that did it the motion of the free bodies.
+template <int NT = PSM_THREADS>
 __device__ __forceinline__ void block_ft_finish(double (*s_ft)[PSM_MAX_BODIES * 6], const StepParams& p) {
-  constexpr int NW = PSM_THREADS / 32;
+  constexpr int NW = NT / 32;
   __shared__ double blk[PSM_MAX_BODIES * 6];
   const int ncomp = p.nbodies * 6;
   __syncthreads();
@@ -1031,7 +1151,12 @@ __device__ __forceinline__ void block_ft_finish(double (*s_ft)[PSM_MAX_BODIES * 
     blk[threadIdx.x] = s;
   }
   __syncthreads();
-  grid_reduce(blk, ncomp, p.partials, p.ticket, p.ft_out);
+  if (grid_reduce<NT>(blk, ncomp, p.partials, p.ticket, p.ft_out) && p.free_mask) {
+    __syncthreads();  // the sums are in ft_out (written by this block)
+    const int warp = threadIdx.x >> 5;
+    for (int b = warp; b < p.nbodies; b += NW)
+      if ((p.free_mask >> b) & 1u) body_update(p.dyn + b, p.dbody + b, p.ft_out + 6 * b, p.g.nx, p.g.ny, p.g.nz);
+  }
 }
 
 // Tile walk of a persistent block: tile index t = (z nty + ty) ntx + tx,
