@@ -364,7 +364,8 @@ int psm_synchronize(psm_handle h);
 
 /* Step-kernel variant: PSM_KERNEL_AUTO (default) uses the TMA-staged kernel
  * for every step the shape allows (the faster variant measured on GB300), else
- * plain global loads;
+ * plain global loads; FP64 grids of at most 256 cells per SM, which the
+ * arithmetic bounds, always take plain loads in smaller blocks;
  * PSM_KERNEL_PLAIN forces plain loads; PSM_KERNEL_TMA forces TMA staging for
  * every step the shape allows (PSM_ERR_UNSUPPORTED if it allows none).  TMA
  * shapes: with TX = min(256, nx): nx % TX == 0, 256 % nx == 0 when nx < 256,
@@ -504,7 +505,8 @@ int psm_check_device_buffer(const void* p, int64_t bytes);
 #define PSM_KERNEL_PLAIN 1
 #define PSM_KERNEL_TMA 2
 int psm_set_kernel_variant(psm_handle h, int variant);
-/* The variant psm_step uses now (PSM_KERNEL_PLAIN or PSM_KERNEL_TMA). */
+/* The variant psm_step uses now (PSM_KERNEL_PLAIN or PSM_KERNEL_TMA; under
+ * PSM_KERNEL_AUTO: PSM_KERNEL_TMA where the shape allows it). */
 int psm_kernel_variant(psm_handle h, int* out);
 
 /* Diagnostics (host only, no GPU needed): the shared-memory layout the

@@ -148,6 +148,33 @@ __device__ __forceinline__ T adj_fluid_cell(const ConstT<T>& C, int solid, T inv
   return bb;
 }
 
+// Tile walk of a persistent block: tile index t = (z nty + ty) ntx + tx,
+// advanced by the grid size without divisions after the first tile.
+struct TileWalk {
+  int tx, ty, z;       // current tile
+  int gx, gy, gz;      // the grid size, decomposed like a tile index
+  int ntx, nty;
+  __device__ __forceinline__ void init(const Tiling& t, int tile, int step) {
+    ntx = t.ntx;
+    nty = t.nty;
+    tx = tile % ntx;
+    ty = (tile / ntx) % nty;
+    z = tile / ntx / nty;
+    gx = step % ntx;
+    gy = (step / ntx) % nty;
+    gz = step / ntx / nty;
+  }
+  __device__ __forceinline__ void advance() {
+    tx += gx;
+    int c = tx >= ntx;
+    tx -= c ? ntx : 0;
+    ty += gy + c;
+    c = ty >= nty;
+    ty -= c ? nty : 0;
+    z += gz + c;
+  }
+};
+
 // PART: 0 every tile; 1 the fluid-only tiles (no scalar sums: a lean kernel
 // that fits three blocks per SM); 2 the general tiles (with the FP64 sums).
 // A step launches 1 and 2 (disjoint cells) or 0.
@@ -526,7 +553,7 @@ __global__ void __launch_bounds__(PSM_THREADS) k_adjoint_init(const __grid_const
 #endif
 template <class S, int Q, int TRT, int PART>
 cudaError_t launch_adjoint_part(const AdjParams& p, cudaStream_t st) {
-  static int blocks = persistent_blocks(k_adjoint<S, Q, TRT, PART>, 1ll << 40);
+  static int blocks = persistent_blocks(k_adjoint<S, Q, TRT, PART>);
   const int grid = (int)(p.t.ntiles < blocks ? p.t.ntiles : blocks);
   k_adjoint<S, Q, TRT, PART><<<grid, PSM_THREADS, 0, st>>>(p);
   return cudaGetLastError();

@@ -606,6 +606,19 @@ bool encode_maps(const psm_solver* h, void* buf, BufMaps& m, const psm::Tiling& 
   return r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS && r3 == CUDA_SUCCESS;
 }
 
+// FP64 storage under PSM_KERNEL_AUTO on a grid of fewer 256-cell blocks than the
+// GPU has SMs: the plain kernel with blocks of 64 cells.  FP64 arithmetic bounds
+// the step (an SM issues one FP64 warp instruction in about 16 clocks), so the
+// cells of a body, the slow ones above all, are spread over four times as many
+// blocks: 32^3 with a sphere 33 us a step, 43 us in blocks of 256 (plain or
+// TMA).  Below FP64 the same split only adds blocks to the load reduction (32^3
+// FP32 12.3 us in blocks of 256, 14.3 us in blocks of 64), and on larger grids
+// every SM has several blocks either way.
+bool fine_grid(const psm_solver* h) {
+  const long long sms = h->max_blocks / (2048 / psm::PSM_THREADS);
+  return h->lat.storage == PSM_FP64 && h->variant == PSM_KERNEL_AUTO && h->g.ncell <= sms * psm::PSM_THREADS;
+}
+
 template <class T>
 void fill_consts(const psm_solver* h, psm::ConstT<T>& c) {
   c.rho0 = (T)h->grid.rho0;
@@ -1267,6 +1280,7 @@ int psm_step(psm_handle h, int n) {
   p.partials = h->d_partials;
   p.ticket = h->d_ticket;
   p.err = h->d_err;
+  p.fine = fine_grid(h);
   for (int k = 0; k < n; ++k) {
     if (h->recording && (h->step - h->rec_n0) % h->rec_K == 0 &&
         (int64_t)h->ckpt.size() == (h->step - h->rec_n0) / h->rec_K) {
@@ -1292,7 +1306,7 @@ int psm_step(psm_handle h, int n) {
     p.dbody = h->d_dev_bodies;
     p.dyn = h->d_dyn;
     // the AA odd step runs with plain loads unless its TMA variant applies
-    const bool tma_now = use_tma && (mode != psm::MODE_AA_ODD ||
+    const bool tma_now = use_tma && !p.fine && (mode != psm::MODE_AA_ODD ||
                                      (h->tma_odd_ok && (h->variant == PSM_KERNEL_TMA || !PSM_AA_ODD_PLAIN)));
     p.t = !tma_now ? h->tiling : (mode == psm::MODE_AA_ODD ? h->tma_tiling_odd : h->tma_tiling);
     psm::TmaMaps tm;

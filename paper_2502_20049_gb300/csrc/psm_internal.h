@@ -215,6 +215,7 @@ struct StepParams {
   unsigned free_mask;
   DevBody* dbody;
   BodyDyn* dyn;  // their state, advanced by the block that sums the loads
+  int fine;      // plain kernel, FP64: blocks of PSM_FINE_THREADS instead of PSM_THREADS
   const float* delta;  // optional additive eps perturbation per cell (nullptr: none)
   // force/torque reduction
   double* partials;      // [gridDim.x][nbodies * 6]
@@ -272,6 +273,7 @@ struct RemapParams {
 };
 
 constexpr int PSM_THREADS = 256;
+constexpr int PSM_FINE_THREADS = 64;
 
 // Caller-owned memory: PSM_OK when p points into device memory of the current
 // device (or managed memory) with at least `bytes` bytes from p to the end of

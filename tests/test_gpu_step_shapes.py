@@ -1,0 +1,61 @@
+"""The step kernels at the edges of their work split: rows shorter and longer
+than a warp's 32 cells, rows with a remainder, one cell, grids on either side of
+the switch to small blocks, and one to four bodies in the load reduction."""
+
+import numpy as np
+import pytest
+
+from paper_2502_20049_gb300 import workloads as W
+
+from helpers import ft_err, perm_lib_to_oracle, run_gpu, run_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__ as g
+
+    g.build()
+
+
+def case(dims, storage, streaming, Q=19, nb=2, fluid="trt", bc_z=1, steps=5, s=2):
+    nx, ny, nz = dims
+    m = min(dims)
+    shapes = [(W.ELLIPSOID, (0.3 * m + 0.6, 0.2 * m + 0.5, 0.2 * m + 0.4), s), (W.SPHERE, (0.15 * m + 0.5,), 3),
+              (W.BOX, (0.7, 0.6, 0.8), 1), (W.SPHERE, (0.9,), 0)]
+    bodies = [W.BodyCase(k, p, sd, (nx * (0.3 + 0.15 * i), ny * 0.5 + 0.1, nz * (0.6 - 0.1 * i)),
+                         omega=(0.01, 0.02, 0.03 * (-1) ** i), v=(0.03, 0.0, 0.0)) for i, (k, p, sd) in enumerate(shapes[:nb])]
+    return W.Case("shapes", nx, ny, nz, Q=Q, storage=storage, streaming=streaming, fluid=fluid, tau=0.65, solid=1,
+                  weighting=1, bc_z=bc_z, u_in=(0.02, -0.01, 0.03), steps=steps, bodies=bodies)
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (1, 5, 3), (31, 3, 4), (32, 4, 3), (33, 5, 7), (63, 2, 9), (65, 6, 5),
+                                  (203, 7, 5), (300, 3, 4), (40, 40, 40)])
+@pytest.mark.parametrize("streaming,bc_z", [("aa", 1), ("aa", 0), ("twogrid", 1)])
+def test_ragged_rows_fp64_match_the_oracle(dims, streaming, bc_z):
+    c = case(dims, "fp64", streaming, bc_z=bc_z, nb=1 + sum(dims) % 4)
+    g, o = run_gpu(c), run_oracle(c)
+    assert np.abs(g["f"] - o["f"][perm_lib_to_oracle(19)]).max() <= 1e-13
+    assert ft_err(g, o) <= 1e-10
+
+
+@pytest.mark.parametrize("dims", [(32, 32, 38), (64, 64, 9), (33, 31, 36), (95, 20, 20)])
+@pytest.mark.parametrize("storage", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("Q,streaming", [(19, "aa"), (27, "aa"), (19, "twogrid")])
+def test_small_blocks_equal_whole_blocks(dims, storage, Q, streaming):
+    """Small grids take blocks of 64 by themselves; forced plain loads keep blocks
+    of 256.  The same cells in the same warps: states bit for bit, loads to the
+    rounding of the FP64 sums' order."""
+    from paper_2502_20049_gb300 import psm
+
+    c = case(dims, storage, streaming, Q=Q, nb=4, steps=6)
+    a, b = psm.Solver.from_case(c), psm.Solver.from_case(c)
+    b.set_kernel_variant("plain")
+    a.step(c.steps)
+    b.step(c.steps)
+    assert np.array_equal(a.get_state(), b.get_state())
+    for k in range(4):
+        fa, fb = a.force_torque(k), b.force_torque(k)
+        # at most nwarps additions of partials whose sizes sum to at most nwarps times the largest total
+        assert np.abs(fa - fb).max() <= 1e-12 * max(1.0, np.abs(fb).max())
