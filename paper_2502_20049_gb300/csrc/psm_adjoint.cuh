@@ -41,7 +41,8 @@ struct AdjParams {
   float dghostf[27][3]; // the same in FP32
   double* partials;
   unsigned int* ticket;
-  double* acc_out;      // [nbodies * 3 + 3]: dJ/d omega per body, dJ/d u_in
+  double* acc_out;      // k_adjoint_init: dJ/d u_in
+  double* slot;         // the blocks' partials of a step's scalar terms (store_slot)
   ConstT<float> cf;
   ConstT<double> cd;
   // slot base pointers (elements): f + i ncell (storage S), lam_in / lam_out + i ncell (T)
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(PSM_THREADS, sizeof(S) == 8 ? 1 : (PART == 1 ?
     blk[threadIdx.x] = s;
   }
   __syncthreads();
-  grid_reduce(blk, ncomp, p.partials, p.ticket, p.acc_out);
+  store_slot(p.slot, blk, ncomp);
 }
 
 // Initial-state term of dJ/d u_in when f^{n0} = f^eq(rho0, u_in) everywhere:

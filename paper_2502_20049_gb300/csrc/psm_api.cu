@@ -149,13 +149,10 @@ struct psm_solver {
   std::vector<BufMaps> rec_maps;
   // a second set of recompute buffers and its stream: psm_backward recomputes
   // the segment before the current one while the adjoint sweeps the current
-  // one (allocated when the device has room; otherwise one set, in sequence);
-  // the recompute's force/torque sums go to their own grid-reduction scratch
+  // one (allocated when the device has room; otherwise one set, in sequence)
   std::vector<void*> rec_slots2;
   std::vector<BufMaps> rec_maps2;
   cudaStream_t rec_stream = nullptr;
-  double* d_partials2 = nullptr;
-  unsigned int* d_ticket2 = nullptr;
   void* rec_lam[2] = {nullptr, nullptr};  // the two adjoint fields
   double* rec_grad = nullptr;             // dJ/d delta accumulator
 };
@@ -512,6 +509,18 @@ bool direct_array(const psm_solver* h, const void* p, size_t bytes, size_t align
   return ok;
 }
 
+// one step's load partials: the block count, then the blocks' sums
+size_t slot_doubles(const psm_solver* h) { return 1 + (size_t)h->max_blocks * PSM_MAX_BODIES * 6; }
+
+// Sum `count` stored slots into rows first, first + dir, ... of out.
+cudaError_t reduce_slots(const psm_solver* h, int count, int ncomp, double* out, int row, int64_t first, int dir,
+                         int64_t cap) {
+  if (count < 1) return cudaSuccess;
+  psm::k_reduce_slots<<<count, psm::PSM_THREADS, 0, h->stream>>>(h->d_partials, (long long)slot_doubles(h), ncomp, out,
+                                                                 row, first, dir, cap);
+  return cudaGetLastError();
+}
+
 int import_uniform(psm_solver* h, double rho, const double u[3]) {
   IoParams p;
   io_base(h, p);
@@ -819,7 +828,7 @@ int create_impl(const psm_grid* grid, const psm_lattice* lattice, const psm_coll
       if (e != cudaSuccess) return cleanup(cuda_fail(e, "PDF buffer allocation"));
     }
   }
-  e = cudaMalloc(&h->d_partials, sizeof(double) * (size_t)h->max_blocks * PSM_MAX_BODIES * 6);
+  e = cudaMalloc(&h->d_partials, sizeof(double) * slot_doubles(h) * psm::PSM_SLOTS);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_ticket, sizeof(unsigned int));
   h->cap = 1 << 16;
   if (e == cudaSuccess) e = cudaMalloc(&h->d_series, sizeof(double) * (size_t)h->cap * PSM_MAX_BODIES * 6);
@@ -899,8 +908,6 @@ int psm_destroy(psm_handle h) {
   for (void* c : h->ckpt) cudaFree(c);
   for (void* c : h->rec_slots) cudaFree(c);
   for (void* c : h->rec_slots2) cudaFree(c);
-  cudaFree(h->d_partials2);
-  cudaFree(h->d_ticket2);
   if (h->rec_stream) cudaStreamDestroy(h->rec_stream);
   cudaFree(h->d_dyn);
   cudaFree(h->d_dev_bodies);
@@ -1281,14 +1288,27 @@ int psm_step(psm_handle h, int n) {
   p.ticket = h->d_ticket;
   p.err = h->d_err;
   p.fine = fine_grid(h);
+  // the loads of several steps in one reduction, unless a free body waits for each
+  const bool later = n > 1 && h->nbodies > 0 && !h->free_mask;
+  int stored = 0;  // slots of the last steps not summed yet
+  auto flush = [&]() {
+    const cudaError_t e = reduce_slots(h, stored, h->nbodies * 6, h->d_series, PSM_MAX_BODIES * 6, h->step - stored, 1,
+                                       h->cap);
+    stored = 0;
+    return e;
+  };
   for (int k = 0; k < n; ++k) {
     if (h->recording && (h->step - h->rec_n0) % h->rec_K == 0 &&
         (int64_t)h->ckpt.size() == (h->step - h->rec_n0) / h->rec_K) {
       const int rc = take_checkpoint(h);
-      if (rc != PSM_OK) return rc;
+      if (rc != PSM_OK) {
+        flush();
+        return rc;
+      }
     }
     for (int b = 0; b < h->nbodies; ++b) p.body[b] = dev_body(h, b, h->step);
     p.ft_out = h->d_series + (size_t)(h->step % h->cap) * PSM_MAX_BODIES * 6;
+    p.ft_slot = later ? h->d_partials + stored * slot_doubles(h) : nullptr;
     int mode, src;
     if (h->lat.streaming == PSM_STREAM_TWO_GRID) {
       mode = psm::MODE_TG;
@@ -1318,10 +1338,19 @@ int psm_step(psm_handle h, int n) {
     }
     cudaError_t e = tma_now ? psm::launch_step_tma(h->lat.storage, h->Q, mode, p, tm, h->stream)
                             : psm::launch_step(h->lat.storage, h->Q, mode, p, h->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+    if (e != cudaSuccess) {
+      flush();
+      return cuda_fail(e, "step kernel launch");
+    }
     if (h->lat.streaming == PSM_STREAM_TWO_GRID) h->cur ^= 1;
     h->step++;
+    if (later && ++stored == psm::PSM_SLOTS) {
+      const cudaError_t r = flush();
+      if (r != cudaSuccess) return cuda_fail(r, "force/torque reduction launch");
+    }
   }
+  const cudaError_t r = flush();
+  if (r != cudaSuccess) return cuda_fail(r, "force/torque reduction launch");
   return PSM_OK;
 }
 
@@ -1341,8 +1370,8 @@ int psm_set_eps_delta(psm_handle h, const float* delta) {
 // Buffers of psm_backward, allocated when recording starts (a one-time cost
 // outside the backward sweep) and kept by the handle: K - 1 recompute states
 // with their tensor maps, two adjoint fields, the gradient accumulator.
-// The second recompute set of psm_backward (K - 1 states, their tensor maps,
-// the recompute stream and its reduction scratch), allocated only while at
+// The second recompute set of psm_backward (K - 1 states, their tensor maps and
+// the recompute stream), allocated only while at
 // least a sixteenth of the device memory stays free; without it psm_backward
 // recomputes and sweeps each segment in turn on the solver's stream.
 static void ensure_second_recompute_set(psm_solver* h, int K) {
@@ -1363,16 +1392,6 @@ static void ensure_second_recompute_set(psm_solver* h, int K) {
     if (ok && h->tma_tg_ok) ok = encode_maps(h, slots[k], maps[k], h->tma_tiling_tg);
   }
   if (ok && !h->rec_stream) ok = cudaStreamCreateWithFlags(&h->rec_stream, cudaStreamNonBlocking) == cudaSuccess;
-  if (ok && !h->d_partials2)
-    ok = cudaMalloc(&h->d_partials2, sizeof(double) * (size_t)h->max_blocks * PSM_MAX_BODIES * 6) == cudaSuccess;
-  if (ok && !h->d_ticket2) {
-    ok = cudaMalloc(&h->d_ticket2, sizeof(unsigned int)) == cudaSuccess;
-    if (ok) ok = cudaMemsetAsync(h->d_ticket2, 0, sizeof(unsigned int), h->stream) == cudaSuccess;
-    if (!ok) {
-      cudaFree(h->d_ticket2);
-      h->d_ticket2 = nullptr;
-    }
-  }
   if (!ok) {
     cudaGetLastError();  // an allocation that failed is not an error of the call
     for (void* c : slots) cudaFree(c);
@@ -1481,14 +1500,12 @@ int psm_backward(psm_handle h, const double* dJ_dFT, double* grad_eps, double* g
   void* lam1 = h->rec_lam[1];
   double* grad = h->rec_grad;
   // small scratch (stream ordered): the weights and the per-step accumulators
-  double *wdev = nullptr, *acc = nullptr, *ftscratch = nullptr;
+  double *wdev = nullptr, *acc = nullptr;
   cudaError_t e = cudaMallocAsync((void**)&wdev, sizeof(double) * w.size(), st);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&acc, sizeof(double) * (size_t)(N + 1) * ncomp, st);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&ftscratch, sizeof(double) * PSM_MAX_BODIES * 6, st);
   auto release = [&]() {
     cudaFreeAsync(wdev, st);
     cudaFreeAsync(acc, st);
-    cudaFreeAsync(ftscratch, st);
   };
   if (e != cudaSuccess) {
     release();
@@ -1512,10 +1529,7 @@ int psm_backward(psm_handle h, const double* dJ_dFT, double* grad_eps, double* g
   sp.weighting = h->col.weighting;
   sp.nbodies = nb;
   sp.delta = h->d_delta;
-  sp.partials = h->d_partials;
-  sp.ticket = h->d_ticket;
-  sp.ft_out = ftscratch;
-  sp.err = h->d_err;
+  sp.err = h->d_err;  // (ft_out, ft_slot null: the recompute wants no loads)
   psm::AdjParams ap;
   std::memset(&ap, 0, sizeof ap);
   ap.g = h->g;
@@ -1554,11 +1568,8 @@ int psm_backward(psm_handle h, const double* dJ_dFT, double* grad_eps, double* g
     if (e == cudaSuccess) e = cudaEventRecord(ev[0], st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(rs, ev[0], 0);
   }
-  StepParams rp = sp;  // the recompute's own reduction scratch when it runs beside the adjoint
-  if (overlap) {
-    rp.partials = h->d_partials2;
-    rp.ticket = h->d_ticket2;
-  }
+  StepParams rp = sp;
+  int stored = 0;  // adjoint steps whose scalar terms are not summed yet
   // recompute f^{ns+1} .. f^{ne-1} of segment m into set q
   auto recompute = [&](int64_t m, int q) {
     if (e != cudaSuccess) return;
@@ -1609,9 +1620,14 @@ int psm_backward(psm_handle h, const double* dJ_dFT, double* grad_eps, double* g
         }
       }
       ap.w = wdev + (size_t)(n - h->rec_n0) * nb * 6;
-      ap.acc_out = acc + (size_t)(n - h->rec_n0) * ncomp;
+      ap.slot = h->d_partials + stored * slot_doubles(h);
       e = launch_adjoint(h->lat.storage, h->Q, ap.trt, ap, st);
       std::swap(la, lb);
+      if (e == cudaSuccess && (++stored == psm::PSM_SLOTS || n == h->rec_n0)) {
+        // the last `stored` steps, n + stored - 1 down to n
+        e = reduce_slots(h, stored, ncomp, acc, ncomp, n - h->rec_n0 + stored - 1, -1, N + 1);
+        stored = 0;
+      }
     }
     if (overlap && e == cudaSuccess) {
       e = cudaEventRecord(ev[3 + q], st);

@@ -221,6 +221,7 @@ struct StepParams {
   double* partials;      // [gridDim.x][nbodies * 6]
   unsigned int* ticket;  // zero between launches
   double* ft_out;        // [nbodies * 6] of this step (body convention)
+  double* ft_slot;       // not null: the blocks' partials go here instead (store_slot); neither: no loads wanted
   int* err;              // set non-zero by a kernel that gave up waiting (never traps)
   ConstT<float> cf;      // constants for FP32 arithmetic
   ConstT<double> cd;     // constants for FP64 arithmetic
@@ -274,6 +275,8 @@ struct RemapParams {
 
 constexpr int PSM_THREADS = 256;
 constexpr int PSM_FINE_THREADS = 64;
+// steps whose load partials are kept for one k_reduce_slots launch
+constexpr int PSM_SLOTS = 16;
 
 // Caller-owned memory: PSM_OK when p points into device memory of the current
 // device (or managed memory) with at least `bytes` bytes from p to the end of

@@ -341,20 +341,53 @@ __device__ __forceinline__ V warp_sum(V v) {
 template <class T>
 using ft_t = typename std::conditional<sizeof(T) == 8, double, float>::type;
 
+// out[c] = sum over the G blocks' partials[j][c], c < ncomp, by one block of NT
+// threads in a fixed order.  Bound by latency: the warps take the components
+// side by side (several share one where there are fewer), and each lane loads
+// up to 16 partials before it adds the first.
+template <int NT>
+__device__ __forceinline__ void sum_partials(const double* partials, int G, int ncomp, double* out) {
+  constexpr int NW = NT / 32;
+  __shared__ double red[NW];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int share = ncomp < NW ? NW / ncomp : 1;  // warps per component
+  for (int c = warp / share; c < ncomp; c += NW / share) {
+    double acc = 0.0;
+    for (int j0 = (warp % share) * 32 + lane; j0 < G; j0 += share * 512) {
+      double v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const int j = j0 + k * share * 32;
+        v[k] = j < G ? __ldcg(&partials[(long long)j * ncomp + c]) : 0.0;
+      }
+#pragma unroll
+      for (int h = 8; h > 0; h >>= 1)
+#pragma unroll
+        for (int k = 0; k < h; ++k) v[k] += v[k + h];
+      acc += v[0];
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) {
+      if (share == 1) out[c] = acc;
+      else red[warp] = acc;
+    }
+  }
+  __syncthreads();
+  if (share > 1 && (int)threadIdx.x < ncomp) {
+    double v = red[threadIdx.x * share];
+    for (int k = 1; k < share; ++k) v += red[threadIdx.x * share + k];
+    out[threadIdx.x] = v;
+  }
+}
+
 // Block-wide ordered reduction of per-block values v[0..ncomp) held in shared
 // memory `blk` into partials[blockIdx.x]; the last block to finish sums all
 // partials in a fixed order into out[0..ncomp) and returns true.  Deterministic
-// for a fixed grid.  The last block's sum is a tail that nothing overlaps, bound
-// by latency: the warps take the components side by side (several warps share
-// one where there are fewer components), four independent chains per lane, and
-// no block barrier between components (one component after the other with a
-// shared-memory tree took 5 us a step with one body, 14 us with two).
+// for a fixed grid.
 template <int NT = PSM_THREADS>
 __device__ __forceinline__ bool grid_reduce(const double* blk, int ncomp, double* partials, unsigned int* ticket,
                                             double* out) {
-  constexpr int NW = NT / 32;
   __shared__ unsigned int s_last;
-  __shared__ double red[NW];
   if ((int)threadIdx.x < ncomp) {
     partials[(long long)blockIdx.x * ncomp + threadIdx.x] = blk[threadIdx.x];
     __threadfence();
@@ -364,32 +397,16 @@ __device__ __forceinline__ bool grid_reduce(const double* blk, int ncomp, double
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = (int)gridDim.x;
-  const int share = ncomp < NW ? NW / ncomp : 1;  // warps per component
-  for (int c = warp / share; c < ncomp; c += NW / share) {
-    const int part = warp % share;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int j = part * 32 + lane; j < G; j += share * 128) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int jj = j + k * share * 32;
-        if (jj < G) a[k] += __ldcg(&partials[(long long)jj * ncomp + c]);
-      }
-    }
-    const double v = warp_sum((a[0] + a[1]) + (a[2] + a[3]));
-    if (lane == 0) {
-      if (share == 1) out[c] = v;
-      else red[warp] = v;
-    }
-  }
-  __syncthreads();
-  if (share > 1 && (int)threadIdx.x < ncomp) {
-    double v = red[threadIdx.x * share];
-    for (int k = 1; k < share; ++k) v += red[threadIdx.x * share + k];
-    out[threadIdx.x] = v;
-  }
+  sum_partials<NT>(partials, (int)gridDim.x, ncomp, out);
   if (threadIdx.x == 0) *ticket = 0u;
   return true;
+}
+
+// The blocks' partials of a kernel whose sum is taken later (k_reduce_slots): the
+// number of blocks, then [block][ncomp].
+__device__ __forceinline__ void store_slot(double* slot, const double* blk, int ncomp) {
+  if ((int)threadIdx.x < ncomp) slot[1 + (long long)blockIdx.x * ncomp + threadIdx.x] = blk[threadIdx.x];
+  if (blockIdx.x == 0 && threadIdx.x == 0) slot[0] = (double)gridDim.x;
 }
 
 // ---------------------------------------------------------------------------
@@ -1129,7 +1146,11 @@ __device__ __forceinline__ void warp_ft(double (*s_ft)[PSM_MAX_BODIES * 6], int 
 }
 
 // Block sum of the per-warp slots (fixed order), then the grid-wide ordered
-// sum, and in the block that did it the motion of the free bodies.
+// sum, and in the block that did it the motion of the free bodies.  The grid
+// sum is a tail of every step that nothing overlaps (fences, a ticket, one
+// block's loads: about 5 us); where no body waits for it, the steps of one call
+// store their partials and k_reduce_slots sums those of up to PSM_SLOTS steps
+// in one launch, in the same order.
 template <int NT = PSM_THREADS>
 __device__ __forceinline__ void block_ft_finish(double (*s_ft)[PSM_MAX_BODIES * 6], const StepParams& p) {
   constexpr int NW = NT / 32;
@@ -1142,6 +1163,10 @@ __device__ __forceinline__ void block_ft_finish(double (*s_ft)[PSM_MAX_BODIES * 
     blk[threadIdx.x] = s;
   }
   __syncthreads();
+  if (p.ft_slot) {
+    store_slot(p.ft_slot, blk, ncomp);
+    return;
+  }
   if (grid_reduce<NT>(blk, ncomp, p.partials, p.ticket, p.ft_out) && p.free_mask) {
     __syncthreads();  // the sums are in ft_out (written by this block)
     const int warp = threadIdx.x >> 5;
@@ -1232,7 +1257,7 @@ __global__ void __launch_bounds__(NT, step_min_blocks<S, Q, FL>() * PSM_THREADS 
   using T = typename Store<S>::T;
   __shared__ double s_ft[NT / 32][PSM_MAX_BODIES * 6];
   __shared__ DevBody s_body[PSM_MAX_BODIES];
-  const int nb = p.nbodies;
+  const int nft = p.ft_out || p.ft_slot ? p.nbodies : 0;  // bodies whose loads are wanted
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int k = lane; k < PSM_MAX_BODIES * 6; k += 32) s_ft[warp][k] = 0.0;
   load_bodies(p, s_body);
@@ -1266,7 +1291,7 @@ __global__ void __launch_bounds__(NT, step_min_blocks<S, Q, FL>() * PSM_THREADS 
         psm_store<S, Q, MODE, GEN>(p, sn, zg, cell, f);
       }
     }
-    if (GEN) warp_ft(s_ft, nb, active && solid_cell && owner >= 0, owner, ft);
+    if (GEN) warp_ft(s_ft, nft, active && solid_cell && owner >= 0, owner, ft);
   };
 
   // this warp's unit and the stride over units, both as (x unit, y, z)
@@ -1289,7 +1314,7 @@ __global__ void __launch_bounds__(NT, step_min_blocks<S, Q, FL>() * PSM_THREADS 
     y -= c ? p.g.ny : 0;
     z += gz + c;
   }
-  if (nb == 0) return;
+  if (nft == 0) return;
   block_ft_finish<NT>(s_ft, p);
 }
 
@@ -1490,7 +1515,7 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
   unsigned long long* empty = full + NST;
   static_assert(2 * NST * 8 <= 128, "stage barriers exceed their 128 bytes");
   constexpr int NW = PSM_THREADS / 32;
-  const int nb = p.nbodies;
+  const int nft = p.ft_out || p.ft_slot ? p.nbodies : 0;  // bodies whose loads are wanted
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int k = lane; k < PSM_MAX_BODIES * 6; k += 32) s_ft[warp][k] = 0.0;
   const int TX = p.t.tx, TY = p.t.ty;
@@ -1681,7 +1706,7 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
         sn.init(p.g, x, y, z, cell);
         psm_store<S, Q, MODE, GEN>(p, sn, zg, cell, f);
       }
-      if (GEN) warp_ft(s_ft, nb, solid_cell && owner >= 0, owner, ft);
+      if (GEN) warp_ft(s_ft, nft, solid_cell && owner >= 0, owner, ft);
     };
     if constexpr (MODE == MODE_AA_EVEN) {
       // only general tiles come here (the fluid-only ones took the pairs above):
@@ -1718,7 +1743,7 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
     }
     __syncthreads();
   }
-  if (nb == 0) return;
+  if (nft == 0) return;
   block_ft_finish(s_ft, p);
 }
 
@@ -2139,6 +2164,15 @@ __global__ void __launch_bounds__(PSM_THREADS) k_mass(const __grid_constant__ Io
   }
   __syncthreads();
   grid_reduce(blk, 1, p.partials, p.ticket, p.sum_out);
+}
+
+// Sums of stored partials (store_slot), one block per slot: slot k into row
+// (first + dir k) mod cap of out (rows of `row` doubles).
+static __global__ void __launch_bounds__(PSM_THREADS) k_reduce_slots(const double* slots, long long slot, int ncomp,
+                                                                     double* out, int row, long long first, int dir,
+                                                                     long long cap) {
+  const double* s = slots + blockIdx.x * slot;
+  sum_partials<PSM_THREADS>(s + 1, (int)s[0], ncomp, out + ((first + dir * (long long)blockIdx.x) % cap) * row);
 }
 
 // ---------------------------------------------------------------------------

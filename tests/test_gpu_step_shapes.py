@@ -59,3 +59,22 @@ def test_small_blocks_equal_whole_blocks(dims, storage, Q, streaming):
         fa, fb = a.force_torque(k), b.force_torque(k)
         # at most nwarps additions of partials whose sizes sum to at most nwarps times the largest total
         assert np.abs(fa - fb).max() <= 1e-12 * max(1.0, np.abs(fb).max())
+
+
+@pytest.mark.parametrize("storage,streaming,dims", [("fp32", "aa", (64, 8, 12)), ("fp16", "twogrid", (33, 9, 7)),
+                                                    ("fp64", "aa", (20, 11, 9))])
+@pytest.mark.parametrize("n", [2, 15, 16, 17, 33])
+def test_loads_of_many_steps_equal_those_of_single_steps(storage, streaming, dims, n):
+    """A call of n steps sums its steps' loads together, a call of one in the step
+    kernel: the same sums bit for bit, around the number of steps summed at once."""
+    from paper_2502_20049_gb300 import psm
+
+    c = case(dims, storage, streaming, nb=3)
+    a, b = psm.Solver.from_case(c), psm.Solver.from_case(c)
+    a.step(n)
+    for _ in range(n):
+        b.step(1)
+    for k in range(3):
+        fa = a.force_torque(k)
+        assert np.abs(fa).max() > 0
+        assert np.array_equal(fa, b.force_torque(k))
