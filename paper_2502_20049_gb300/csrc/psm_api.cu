@@ -512,13 +512,14 @@ bool direct_array(const psm_solver* h, const void* p, size_t bytes, size_t align
 // one step's load partials: the block count, then the blocks' sums
 size_t slot_doubles(const psm_solver* h) { return 1 + (size_t)h->max_blocks * PSM_MAX_BODIES * 6; }
 
-// Sum `count` stored slots into rows first, first + dir, ... of out.
+// Sum `count` stored slots into rows first, first + dir, ... of out, and advance
+// the bodies of free_mask under them.
 cudaError_t reduce_slots(const psm_solver* h, int count, int ncomp, double* out, int row, int64_t first, int dir,
-                         int64_t cap) {
+                         int64_t cap, unsigned free_mask = 0) {
   if (count < 1) return cudaSuccess;
-  psm::k_reduce_slots<<<count, psm::PSM_THREADS, 0, h->stream>>>(h->d_partials, (long long)slot_doubles(h), ncomp, out,
-                                                                 row, first, dir, cap);
-  return cudaGetLastError();
+  return psm::launch_overlapped(psm::k_reduce_slots, count, psm::PSM_THREADS, 0, h->stream, h->d_partials,
+                                (long long)slot_doubles(h), ncomp, out, row, (long long)first, dir, (long long)cap,
+                                free_mask, h->d_dyn, h->d_dev_bodies, h->g.nx, h->g.ny, h->g.nz);
 }
 
 int import_uniform(psm_solver* h, double rho, const double u[3]) {
@@ -1284,16 +1285,14 @@ int psm_step(psm_handle h, int n) {
   p.weighting = h->col.weighting;
   p.nbodies = h->nbodies;
   p.delta = h->d_delta;
-  p.partials = h->d_partials;
-  p.ticket = h->d_ticket;
   p.err = h->d_err;
   p.fine = fine_grid(h);
-  // the loads of several steps in one reduction, unless a free body waits for each
-  const bool later = n > 1 && h->nbodies > 0 && !h->free_mask;
+  // the loads of up to PSM_SLOTS steps in one reduction; of each where a free body waits for them
+  const int slots = h->free_mask ? 1 : psm::PSM_SLOTS;
   int stored = 0;  // slots of the last steps not summed yet
   auto flush = [&]() {
     const cudaError_t e = reduce_slots(h, stored, h->nbodies * 6, h->d_series, PSM_MAX_BODIES * 6, h->step - stored, 1,
-                                       h->cap);
+                                       h->cap, h->free_mask);
     stored = 0;
     return e;
   };
@@ -1307,8 +1306,8 @@ int psm_step(psm_handle h, int n) {
       }
     }
     for (int b = 0; b < h->nbodies; ++b) p.body[b] = dev_body(h, b, h->step);
-    p.ft_out = h->d_series + (size_t)(h->step % h->cap) * PSM_MAX_BODIES * 6;
-    p.ft_slot = later ? h->d_partials + stored * slot_doubles(h) : nullptr;
+    p.nft = h->nbodies;
+    p.ft_slot = h->d_partials + stored * slot_doubles(h);
     int mode, src;
     if (h->lat.streaming == PSM_STREAM_TWO_GRID) {
       mode = psm::MODE_TG;
@@ -1324,7 +1323,6 @@ int psm_step(psm_handle h, int n) {
     psm::set_slots(p, h->lat.storage, h->Q);
     p.free_mask = h->free_mask;
     p.dbody = h->d_dev_bodies;
-    p.dyn = h->d_dyn;
     // the AA odd step runs with plain loads unless its TMA variant applies
     const bool tma_now = use_tma && !p.fine && (mode != psm::MODE_AA_ODD ||
                                      (h->tma_odd_ok && (h->variant == PSM_KERNEL_TMA || !PSM_AA_ODD_PLAIN)));
@@ -1344,7 +1342,7 @@ int psm_step(psm_handle h, int n) {
     }
     if (h->lat.streaming == PSM_STREAM_TWO_GRID) h->cur ^= 1;
     h->step++;
-    if (later && ++stored == psm::PSM_SLOTS) {
+    if (h->nbodies && ++stored == slots) {
       const cudaError_t r = flush();
       if (r != cudaSuccess) return cuda_fail(r, "force/torque reduction launch");
     }
@@ -1529,7 +1527,7 @@ int psm_backward(psm_handle h, const double* dJ_dFT, double* grad_eps, double* g
   sp.weighting = h->col.weighting;
   sp.nbodies = nb;
   sp.delta = h->d_delta;
-  sp.err = h->d_err;  // (ft_out, ft_slot null: the recompute wants no loads)
+  sp.err = h->d_err;  // (nft 0: the recompute wants no loads)
   psm::AdjParams ap;
   std::memset(&ap, 0, sizeof ap);
   ap.g = h->g;

@@ -213,15 +213,11 @@ struct StepParams {
   // bodies whose motion the device integrates (two-way coupling): bit b set ->
   // body b of this step is dbody[b] (device memory), not body[b]
   unsigned free_mask;
-  DevBody* dbody;
-  BodyDyn* dyn;  // their state, advanced by the block that sums the loads
+  const DevBody* dbody;
   int fine;      // plain kernel, FP64: blocks of PSM_FINE_THREADS instead of PSM_THREADS
   const float* delta;  // optional additive eps perturbation per cell (nullptr: none)
-  // force/torque reduction
-  double* partials;      // [gridDim.x][nbodies * 6]
-  unsigned int* ticket;  // zero between launches
-  double* ft_out;        // [nbodies * 6] of this step (body convention)
-  double* ft_slot;       // not null: the blocks' partials go here instead (store_slot); neither: no loads wanted
+  int nft;          // bodies whose loads are wanted: nbodies, or 0 (the recompute of the backward pass)
+  double* ft_slot;  // the blocks' partial loads (block_ft_finish, k_reduce_slots)
   int* err;              // set non-zero by a kernel that gave up waiting (never traps)
   ConstT<float> cf;      // constants for FP32 arithmetic
   ConstT<double> cd;     // constants for FP64 arithmetic
