@@ -426,13 +426,23 @@ __device__ __forceinline__ void store_slot(double* slot, const double* blk, int 
 #ifndef PSM_MIN_BLOCKS_CUM
 #define PSM_MIN_BLOCKS_CUM 2
 #endif
-// The D3Q27 AA odd step in 2-byte storage (one cell per thread) fits 80
-// registers without spills and runs three blocks, where its even step (two
-// cells per thread) needs the 128-register budget of two.
+// The AA odd step of the TMA kernel in 2-byte storage with BGK/TRT
+// (odd_pairs) holds two cells per thread: two blocks (128 registers).  It is
+// bound by instruction issue: with one cell per thread 545 warp instructions per
+// 32 cells (D3Q19), with x-neighbour pairs, whose shared accesses, stores,
+// addresses and tile bookkeeping serve two cells, 343.  The pairs keep the
+// tiles of one 256-cell row (two-row tiles halved the pipeline's depth): a tile
+// is four warps' work, and the block's two groups of warps take alternate
+// tiles.  1024x1024x960 D3Q19 FP16 14.11 -> 13.67 ms per AA step (even and odd
+// averaged), 512x512x640 D3Q27 3.456 -> 3.348.
+template <class S, int FL, int MODE>
+__host__ __device__ constexpr bool odd_pairs() {
+  return sizeof(S) == 2 && FL != 2 && MODE == MODE_AA_ODD;
+}
 template <class S, int Q, int FL = 0, int MODE = -1>
 __host__ __device__ constexpr int step_min_blocks() {
   if (FL == 2) return sizeof(S) == 8 ? 1 : PSM_MIN_BLOCKS_CUM;
-  if (Q == 27 && sizeof(S) == 2 && MODE == MODE_AA_ODD) return 3;
+  if (odd_pairs<S, FL, MODE>()) return 2;
   return sizeof(S) == 8 ? (Q == 19 ? PSM_MIN_BLOCKS_Q19 - 1 : PSM_MIN_BLOCKS_Q27 - 1)
                         : (Q == 19 ? PSM_MIN_BLOCKS_Q19 : PSM_MIN_BLOCKS_Q27);
 }
@@ -1360,7 +1370,8 @@ struct TmaLayout {
 // st.global; the AA even step stores to the own cells' swapped slots (with
 // two cells per thread, the fluid-only tiles' x-neighbour pairs with one
 // 32-bit access per slot), or, built with PSM_TMA_STORE, through one TMA
-// tensor store per warp.  No block barrier inside the tile loop.
+// tensor store per warp.  In the paired AA odd step (odd_pairs) a tile is the
+// work of every other warp of the block.  No block barrier inside the tile loop.
 // ---------------------------------------------------------------------------
 template <class S, int Q, int MODE, int FL>
 __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>())
@@ -1392,6 +1403,12 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
   unsigned long long* empty = full + NST;
   static_assert(2 * NST * 8 <= 128, "stage barriers exceed their 128 bytes");
   constexpr int NW = PSM_THREADS / 32;
+  // tiles in flight per block: in the paired AA odd step the even warps take the
+  // block's even tiles and the odd warps its odd ones, two x-neighbour cells per
+  // thread; otherwise all warps share each tile
+  constexpr bool PAIRS = odd_pairs<S, FL, MODE>();
+  constexpr int GROUPS = PAIRS ? 2 : 1;
+  static_assert(GROUPS == 1 || LAG % GROUPS == 0, "a warp refills stages that its own group has read");
   const int nb = p.nft;  // bodies whose loads are wanted
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int k = lane; k < PSM_MAX_BODIES * 6; k += 32) s_ft[warp][k] = 0.0;
@@ -1412,7 +1429,7 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
     s_abort = 0;
     for (int s = 0; s < NST; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], NW);
+      mbar_init(&empty[s], NW / GROUPS);
       s_issued[s] = 0;
     }
     fence_mbar_init();
@@ -1543,9 +1560,54 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
         *reinterpret_cast<unsigned*>(static_cast<S*>(p.dst_slot[lat_opp(i)]) + cell) = Pair16<S>::pack(f0[i], f1[i]);
       return;
     }
-    // the thread's cells r = 0 .. CPT-1: (lx, ly + r TYB), one after the other
+    if constexpr (PAIRS && !GEN) {
+      // cells x = hd.x + 2 tg (even) and x + 1: where c_x = 0 one 32-bit shared
+      // load and one 32-bit store serve both
+      const int tg = (warp >> 1) * 32 + lane;
+      T f0[Q], f1[Q];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const unsigned char* row = st + i * L::ROW + 128;
+        if (lat_cx(i) == 0) {
+          Pair16<S>::unpack(reinterpret_cast<const unsigned*>(row)[tg], f0[i], f1[i]);
+        } else {
+          const S* e = reinterpret_cast<const S*>(row) + (2 * tg - lat_cx(i));
+          f0[i] = Store<S>::ld(e);
+          f1[i] = Store<S>::ld(e + 1);
+        }
+      }
+      stage_read(tile, k, s);
+      fluid_collide<T, Q, FL>(p, f0);
+      fluid_collide<T, Q, FL>(p, f1);
+      const int x = hd.x + 2 * tg, y = hd.y;
+      const unsigned cell = ((unsigned)z * (unsigned)p.g.ny + (unsigned)y) * (unsigned)p.g.nx + (unsigned)x;
+      Stencil sn;
+      sn.init(p.g, x, y, z, cell);
+      // x + 2 of the second cell wraps at the row's end (x + 1 of the first never does)
+      const unsigned dx2 = x + 2 == p.g.nx ? 0u - (unsigned)x : 2u;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const int cx = lat_cx(i), cy = lat_cy(i), cz = lat_cz(i);
+        S* d = static_cast<S*>(p.dst_slot[i]);
+        const unsigned r = sn.at(0, cy, cz);
+        if (cx == 0) {
+          *reinterpret_cast<unsigned*>(d + r) = Pair16<S>::pack(f0[i], f1[i]);
+        } else if (cx > 0) {
+          Store<S>::st(d + (unsigned)(r + 1u), f0[i]);
+          Store<S>::st(d + (unsigned)(r + dx2), f1[i]);
+        } else {
+          Store<S>::st(d + (unsigned)(r + sn.dx[0]), f0[i]);
+          Store<S>::st(d + r, f1[i]);
+        }
+      }
+      return;
+    }
+    // the thread's cells r = 0 .. CELLS-1: (lx, ly + r TYB), one after the other
+    // (paired AA odd step: 128 cells of the row apart, so that a warp's lanes are x neighbours)
+    constexpr int CELLS = PAIRS ? 2 : CPT;
     auto one_cell = [&](int r) {
-      const int x = hd.x + lx, y = hd.y + ly + r * TYB;
+      const int xl = PAIRS ? (warp >> 1) * 32 + lane + r * (PSM_THREADS / 2) : lx;
+      const int x = hd.x + xl, y = hd.y + (PAIRS ? 0 : ly + r * TYB);
       const unsigned cell = ((unsigned)z * (unsigned)p.g.ny + (unsigned)y) * (unsigned)p.g.nx + (unsigned)x;
       T f[Q];
 #pragma unroll
@@ -1555,10 +1617,10 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
         } else if (L::LOAD_OWN) {
           f[i] = Store<S>::ld(reinterpret_cast<const S*>(st) + (i * CPT + r) * PSM_THREADS + threadIdx.x);
         } else {
-          f[i] = Store<S>::ld(reinterpret_cast<const S*>(st + i * L::ROW + 128) + (lx - lat_cx(i)));
+          f[i] = Store<S>::ld(reinterpret_cast<const S*>(st + i * L::ROW + 128) + (xl - lat_cx(i)));
         }
       }
-      if (r == CPT - 1) stage_read(tile, k, s);
+      if (r == CELLS - 1) stage_read(tile, k, s);
       int owner = -1;
       bool solid_cell = false;
       ft_t<T> ft[6] = {0, 0, 0, 0, 0, 0};
@@ -1587,19 +1649,19 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
       }
       if (GEN) warp_ft(s_ft, nb, solid_cell && owner >= 0, owner, ft);
     };
-    if constexpr (MODE == MODE_AA_EVEN) {
+    if constexpr (MODE == MODE_AA_EVEN || PAIRS) {
       // only general tiles come here (the fluid-only ones took the pairs above):
       // one copy of the PSM code
 #pragma unroll 1
-      for (int r = 0; r < CPT; ++r) one_cell(r);
+      for (int r = 0; r < CELLS; ++r) one_cell(r);
     } else {
 #pragma unroll
-      for (int r = 0; r < CPT; ++r) one_cell(r);
+      for (int r = 0; r < CELLS; ++r) one_cell(r);
     }
   };
 
-  int k = 0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+  int k = GROUPS == 1 ? 0 : warp % GROUPS;
+  for (int tile = blockIdx.x + k * gridDim.x; tile < ntiles; tile += GROUPS * gridDim.x, k += GROUPS) {
     const int s = k % NST;
     // bounded wait for the stage, warp-uniform outcome (on time-out the block's
     // results are invalid: s_abort; the warp leaves the loop)
