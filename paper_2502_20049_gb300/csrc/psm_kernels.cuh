@@ -426,23 +426,26 @@ __device__ __forceinline__ void store_slot(double* slot, const double* blk, int 
 #ifndef PSM_MIN_BLOCKS_CUM
 #define PSM_MIN_BLOCKS_CUM 2
 #endif
-// The AA odd step of the TMA kernel in 2-byte storage with BGK/TRT
-// (odd_pairs) holds two cells per thread: two blocks (128 registers).  It is
-// bound by instruction issue: with one cell per thread 545 warp instructions per
-// 32 cells (D3Q19), with x-neighbour pairs, whose shared accesses, stores,
-// addresses and tile bookkeeping serve two cells, 343.  The pairs keep the
-// tiles of one 256-cell row (two-row tiles halved the pipeline's depth): a tile
-// is four warps' work, and the block's two groups of warps take alternate
-// tiles.  1024x1024x960 D3Q19 FP16 14.11 -> 13.67 ms per AA step (even and odd
-// averaged), 512x512x640 D3Q27 3.456 -> 3.348.
+// Tiles of 256 cells with two x neighbours per thread (TMA kernel, 2-byte
+// storage): a tile is four warps' work, and the block's two groups of warps take
+// alternate tiles.  These steps are bound by instruction issue, and a pair shares
+// shared-memory accesses, stores, addresses and the tile's bookkeeping.
+//   AA odd, BGK/TRT: 545 -> 343 warp instructions per 32 cells (D3Q19).  Two-row
+//     tiles for the pairs halved the pipeline's depth; one-row tiles keep it.
+//     1024x1024x960 D3Q19 FP16 14.11 -> 13.67 ms per AA step (even and odd
+//     averaged), 512x512x640 D3Q27 3.456 -> 3.348.
+//   Cumulant, every mode: the additions and multiply-adds of its arithmetic
+//     (about 240 of 449 instructions per 32 cells) are packed FP32 instructions
+//     as well; 128 registers without spills.  256^3 FP16 AA 296.8 -> 245.6 us a
+//     step, two-grid 289.6 -> 242.1 (pairs alone: 277.5 and 274.4).
 template <class S, int FL, int MODE>
-__host__ __device__ constexpr bool odd_pairs() {
-  return sizeof(S) == 2 && FL != 2 && MODE == MODE_AA_ODD;
+__host__ __device__ constexpr bool tile_pairs() {
+  return sizeof(S) == 2 && MODE >= 0 && (FL == 2 || MODE == MODE_AA_ODD);
 }
 template <class S, int Q, int FL = 0, int MODE = -1>
 __host__ __device__ constexpr int step_min_blocks() {
   if (FL == 2) return sizeof(S) == 8 ? 1 : PSM_MIN_BLOCKS_CUM;
-  if (odd_pairs<S, FL, MODE>()) return 2;
+  if (tile_pairs<S, FL, MODE>()) return 2;
   return sizeof(S) == 8 ? (Q == 19 ? PSM_MIN_BLOCKS_Q19 - 1 : PSM_MIN_BLOCKS_Q27 - 1)
                         : (Q == 19 ? PSM_MIN_BLOCKS_Q19 : PSM_MIN_BLOCKS_Q27);
 }
@@ -505,6 +508,43 @@ __device__ __forceinline__ T r_div(T a, T b) {
   if constexpr (sizeof(T) == 4) return __fdiv_rn(a, b);
   else return __ddiv_rn(a, b);
 }
+
+// Two cells' FP32 values side by side: the packed FP32 instructions compute both
+// with one issue, each lane rounded as the scalar operation.
+struct F2 {
+  float2 v;
+  __device__ __forceinline__ F2() {}
+  __device__ __forceinline__ F2(float a) : v(make_float2(a, a)) {}
+  __device__ __forceinline__ F2(float a, float b) : v(make_float2(a, b)) {}
+  __device__ __forceinline__ F2(float2 a) : v(a) {}
+};
+__device__ __forceinline__ F2 operator-(F2 a) { return F2(-a.v.x, -a.v.y); }
+// Additions and fused multiply-adds are packed; multiplications stay scalar: the
+// assembler contracts a packed one into the addition that follows it, its .rn
+// notwithstanding (which would round otherwise than the scalar kernels).
+__device__ __forceinline__ unsigned long long f2_bits(F2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.v.x), "f"(a.v.y));
+  return r;
+}
+__device__ __forceinline__ F2 f2_of(unsigned long long b) {
+  F2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.v.x), "=f"(r.v.y) : "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 r_add(F2 a, F2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ F2 r_mul(F2 a, F2 b) { return F2(__fmul_rn(a.v.x, b.v.x), __fmul_rn(a.v.y, b.v.y)); }
+__device__ __forceinline__ F2 r_fma(F2 a, F2 b, F2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+  return f2_of(r);
+}
+__device__ __forceinline__ F2 r_sub(F2 a, F2 b) { return r_fma(b, F2(-1.0f), a); }  // a - b, rounded once
+__device__ __forceinline__ F2 recip(F2 r) { return F2(recip(r.v.x), recip(r.v.y)); }
 
 // Density deviation, density and velocity of one cell from its shifted PDFs,
 // summed over opposite pairs (i, i + 1): drho = f_0 + sum (f_i + f_i+1),
@@ -575,11 +615,12 @@ __device__ __forceinline__ T feq_shifted_r(int i, T drho, T rho, T vx, T vy, T v
 // The products of omega+-, the weight and the numeric factors are host
 // constants per weight class (ConstT pw, pk, pd); f_i and f_j are not needed
 // once s and d are formed.
-template <class T, bool UNIT>
-__device__ __forceinline__ void cumulant_relax(const ConstT<T>& C, T (&f)[19], T drho, T rho, T ux, T uy, T uz);
+// (T: float, double, or F2 with the float constants)
+template <class T, bool UNIT, class CT>
+__device__ __forceinline__ void cumulant_relax(const CT& C, T (&f)[19], T drho, T rho, T ux, T uy, T uz);
 
-template <class T, int Q, int FL>
-__device__ __forceinline__ void fluid_relax(const ConstT<T>& C, T (&f)[Q], T drho, T rho, T ux, T uy, T uz, T uu) {
+template <class T, int Q, int FL, class CT>
+__device__ __forceinline__ void fluid_relax(const CT& C, T (&f)[Q], T drho, T rho, T ux, T uy, T uz, T uu) {
   if constexpr (FL == 2) {
     static_assert(Q == 19, "the cumulant operator is defined for D3Q19");
     if (C.cum_unit) cumulant_relax<T, true>(C, f, drho, rho, ux, uy, uz);
@@ -629,8 +670,8 @@ __device__ __forceinline__ void fluid_relax(const ConstT<T>& C, T (&f)[Q], T drh
 //     f(s, 0, 0) = ((m_200 - m_220 - m_202) + s (m_100 - m_120 - m_102)) / 2,
 //     f_0 = m_000 - m_200 - m_020 - m_002 + m_220 + m_202 + m_022.
 // Operations are separately rounded (same bits in every kernel that inlines it).
-template <class T, bool UNIT>
-__device__ __forceinline__ void cumulant_relax(const ConstT<T>& C, T (&f)[19], T drho, T rho, T ux, T uy, T uz) {
+template <class T, bool UNIT, class CT>
+__device__ __forceinline__ void cumulant_relax(const CT& C, T (&f)[19], T drho, T rho, T ux, T uy, T uz) {
   auto ad = [](T a, T b) { return r_add(a, b); };
   auto sb = [](T a, T b) { return r_sub(a, b); };
   auto ml = [](T a, T b) { return r_mul(a, b); };
@@ -1120,6 +1161,27 @@ __device__ __forceinline__ void fluid_collide(const StepParams& p, T (&f)[Q]) {
   fluid_relax<T, Q, FL>(C, f, drho, rho, ux, uy, uz, uu);
 }
 
+// Two cells of fluid-only tiles: the cumulant in packed FP32 instructions (see
+// tile_pairs), BGK and TRT one cell after the other, the same bits either way
+// (packed, D3Q19 took 13.85 ms at 1024x1024x960, one by one 13.67, and D3Q27 was
+// no faster).
+template <int Q, int FL>
+__device__ __forceinline__ void fluid_collide2(const StepParams& p, F2 (&f)[Q]) {
+  if constexpr (FL == 2) {
+    F2 drho, rho, ux, uy, uz, uu;
+    moments<F2, Q>(f, F2(p.cf.rho0), drho, rho, ux, uy, uz, uu);
+    fluid_relax<F2, Q, FL>(p.cf, f, drho, rho, ux, uy, uz, uu);
+  } else {
+    float a[Q], b[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) a[i] = f[i].v.x, b[i] = f[i].v.y;
+    fluid_collide<float, Q, FL>(p, a);
+    fluid_collide<float, Q, FL>(p, b);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = F2(a[i], b[i]);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // The fused step kernel with plain global loads, any grid shape.  A warp's unit
 // of work is 32 neighbouring cells of one row (the last unit of a row holds the
@@ -1370,8 +1432,8 @@ struct TmaLayout {
 // st.global; the AA even step stores to the own cells' swapped slots (with
 // two cells per thread, the fluid-only tiles' x-neighbour pairs with one
 // 32-bit access per slot), or, built with PSM_TMA_STORE, through one TMA
-// tensor store per warp.  In the paired AA odd step (odd_pairs) a tile is the
-// work of every other warp of the block.  No block barrier inside the tile loop.
+// tensor store per warp.  With tile_pairs a tile is the work of every other warp
+// of the block.  No block barrier inside the tile loop.
 // ---------------------------------------------------------------------------
 template <class S, int Q, int MODE, int FL>
 __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>())
@@ -1403,10 +1465,9 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
   unsigned long long* empty = full + NST;
   static_assert(2 * NST * 8 <= 128, "stage barriers exceed their 128 bytes");
   constexpr int NW = PSM_THREADS / 32;
-  // tiles in flight per block: in the paired AA odd step the even warps take the
-  // block's even tiles and the odd warps its odd ones, two x-neighbour cells per
-  // thread; otherwise all warps share each tile
-  constexpr bool PAIRS = odd_pairs<S, FL, MODE>();
+  // tile_pairs: the even warps take the block's even tiles and the odd warps its
+  // odd ones, two x-neighbour cells per thread; otherwise all warps share each tile
+  constexpr bool PAIRS = tile_pairs<S, FL, MODE>();
   constexpr int GROUPS = PAIRS ? 2 : 1;
   static_assert(GROUPS == 1 || LAG % GROUPS == 0, "a warp refills stages that its own group has read");
   const int nb = p.nft;  // bodies whose loads are wanted
@@ -1547,39 +1608,40 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
     constexpr bool XPAIR = !GEN && CPT == 2 && MODE == MODE_AA_EVEN && sizeof(S) == 2 && FL != 2 && !L::STORE_TMA;
     if constexpr (XPAIR) {
       const unsigned* sw = reinterpret_cast<const unsigned*>(st) + (py * TX) / 2 + px;
-      T f0[Q], f1[Q];
+      F2 f[Q];
 #pragma unroll
-      for (int i = 0; i < Q; ++i) Pair16<S>::unpack(sw[i * (CPT * PSM_THREADS / 2)], f0[i], f1[i]);
+      for (int i = 0; i < Q; ++i) Pair16<S>::unpack(sw[i * (CPT * PSM_THREADS / 2)], f[i].v.x, f[i].v.y);
       stage_read(tile, k, s);
-      fluid_collide<T, Q, FL>(p, f0);
-      fluid_collide<T, Q, FL>(p, f1);
+      fluid_collide2<Q, FL>(p, f);
       const int x = hd.x + 2 * px, y = hd.y + py;
       const unsigned cell = ((unsigned)z * (unsigned)p.g.ny + (unsigned)y) * (unsigned)p.g.nx + (unsigned)x;
 #pragma unroll
       for (int i = 0; i < Q; ++i)
-        *reinterpret_cast<unsigned*>(static_cast<S*>(p.dst_slot[lat_opp(i)]) + cell) = Pair16<S>::pack(f0[i], f1[i]);
+        *reinterpret_cast<unsigned*>(static_cast<S*>(p.dst_slot[lat_opp(i)]) + cell) = Pair16<S>::pack(f[i].v.x, f[i].v.y);
       return;
     }
     if constexpr (PAIRS && !GEN) {
-      // cells x = hd.x + 2 tg (even) and x + 1: where c_x = 0 one 32-bit shared
-      // load and one 32-bit store serve both
-      const int tg = (warp >> 1) * 32 + lane;
-      T f0[Q], f1[Q];
+      // x neighbours, x even: where c_x = 0 one 32-bit shared load and one 32-bit
+      // store serve both
+      const int tg = (warp >> 1) * 32 + lane, xl = 2 * tg % TX;
+      F2 f[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        const unsigned char* row = st + i * L::ROW + 128;
-        if (lat_cx(i) == 0) {
-          Pair16<S>::unpack(reinterpret_cast<const unsigned*>(row)[tg], f0[i], f1[i]);
+        if (L::LOAD_OWN) {
+          Pair16<S>::unpack(reinterpret_cast<const unsigned*>(st)[i * (PSM_THREADS / 2) + tg], f[i].v.x, f[i].v.y);
         } else {
-          const S* e = reinterpret_cast<const S*>(row) + (2 * tg - lat_cx(i));
-          f0[i] = Store<S>::ld(e);
-          f1[i] = Store<S>::ld(e + 1);
+          const unsigned char* row = st + i * L::ROW + 128;
+          if (lat_cx(i) == 0) {
+            Pair16<S>::unpack(reinterpret_cast<const unsigned*>(row)[tg], f[i].v.x, f[i].v.y);
+          } else {
+            const S* e = reinterpret_cast<const S*>(row) + (2 * tg - lat_cx(i));
+            f[i].v = make_float2(Store<S>::ld(e), Store<S>::ld(e + 1));
+          }
         }
       }
       stage_read(tile, k, s);
-      fluid_collide<T, Q, FL>(p, f0);
-      fluid_collide<T, Q, FL>(p, f1);
-      const int x = hd.x + 2 * tg, y = hd.y;
+      fluid_collide2<Q, FL>(p, f);
+      const int x = hd.x + xl, y = hd.y + 2 * tg / TX;
       const unsigned cell = ((unsigned)z * (unsigned)p.g.ny + (unsigned)y) * (unsigned)p.g.nx + (unsigned)x;
       Stencil sn;
       sn.init(p.g, x, y, z, cell);
@@ -1588,26 +1650,32 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         const int cx = lat_cx(i), cy = lat_cy(i), cz = lat_cz(i);
+        if (MODE == MODE_AA_EVEN) {
+          *reinterpret_cast<unsigned*>(static_cast<S*>(p.dst_slot[lat_opp(i)]) + cell) =
+              Pair16<S>::pack(f[i].v.x, f[i].v.y);
+          continue;
+        }
         S* d = static_cast<S*>(p.dst_slot[i]);
         const unsigned r = sn.at(0, cy, cz);
         if (cx == 0) {
-          *reinterpret_cast<unsigned*>(d + r) = Pair16<S>::pack(f0[i], f1[i]);
+          *reinterpret_cast<unsigned*>(d + r) = Pair16<S>::pack(f[i].v.x, f[i].v.y);
         } else if (cx > 0) {
-          Store<S>::st(d + (unsigned)(r + 1u), f0[i]);
-          Store<S>::st(d + (unsigned)(r + dx2), f1[i]);
+          Store<S>::st(d + (unsigned)(r + 1u), f[i].v.x);
+          Store<S>::st(d + (unsigned)(r + dx2), f[i].v.y);
         } else {
-          Store<S>::st(d + (unsigned)(r + sn.dx[0]), f0[i]);
-          Store<S>::st(d + r, f1[i]);
+          Store<S>::st(d + (unsigned)(r + sn.dx[0]), f[i].v.x);
+          Store<S>::st(d + r, f[i].v.y);
         }
       }
       return;
     }
     // the thread's cells r = 0 .. CELLS-1: (lx, ly + r TYB), one after the other
-    // (paired AA odd step: 128 cells of the row apart, so that a warp's lanes are x neighbours)
+    // (paired: 128 cells of the tile apart, so that a warp's lanes are x neighbours)
     constexpr int CELLS = PAIRS ? 2 : CPT;
     auto one_cell = [&](int r) {
-      const int xl = PAIRS ? (warp >> 1) * 32 + lane + r * (PSM_THREADS / 2) : lx;
-      const int x = hd.x + xl, y = hd.y + (PAIRS ? 0 : ly + r * TYB);
+      const int c = PAIRS ? (warp >> 1) * 32 + lane + r * (PSM_THREADS / 2) : (int)threadIdx.x;
+      const int xl = PAIRS ? c % TX : lx;
+      const int x = hd.x + xl, y = hd.y + (PAIRS ? c / TX : ly + r * TYB);
       const unsigned cell = ((unsigned)z * (unsigned)p.g.ny + (unsigned)y) * (unsigned)p.g.nx + (unsigned)x;
       T f[Q];
 #pragma unroll
@@ -1615,7 +1683,7 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
         if (GEN && zg.from(lat_cz(i))) {
           f[i] = cst<T>(p).ghost[i];
         } else if (L::LOAD_OWN) {
-          f[i] = Store<S>::ld(reinterpret_cast<const S*>(st) + (i * CPT + r) * PSM_THREADS + threadIdx.x);
+          f[i] = Store<S>::ld(reinterpret_cast<const S*>(st) + (PAIRS ? i : i * CPT + r) * PSM_THREADS + c);
         } else {
           f[i] = Store<S>::ld(reinterpret_cast<const S*>(st + i * L::ROW + 128) + (xl - lat_cx(i)));
         }
