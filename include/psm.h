@@ -14,7 +14,9 @@
  *   4. streaming f_i(x + c_i, t + 1) = f*_i(x) (Eq. 1): AA pattern in place, or
  *      two grids,
  *   5. the force and torque on every body (Eq. 10 and Eq. 11), reduced in FP64.
- * It runs fused in one kernel launch per step.
+ * It runs fused in one kernel launch per step; the loads of step 5 are summed
+ * over the blocks by one small launch for up to 16 steps of a call (every step
+ * where a free body moves under them).
  *
  * Conventions:
  *   - lattice units dx = dt = 1; cell (x, y, z) has its centre at
@@ -334,7 +336,7 @@ int psm_body_state(psm_handle h, int body, double* out);
 int psm_set_remap(psm_handle h, int every_step);
 
 /* Run n >= 0 time steps asynchronously on the handle's stream (one fused
- * kernel launch per step; no host synchronisation).  One step is the pose and
+ * kernel launch per step and the sums of the loads; no host synchronisation).  One step is the pose and
  * remap of Sec. 3, the PSM collision Eq. 4 (with Eq. 2/3, Eq. 5/6, Eq. 7-9),
  * streaming Eq. 1 and the force/torque sums Eq. 10/11, in that order. */
 int psm_step(psm_handle h, int n);

@@ -837,6 +837,8 @@ int create_impl(const psm_grid* grid, const psm_lattice* lattice, const psm_coll
   if (e == cudaSuccess) e = cudaMalloc(&h->d_err, sizeof(int));
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "scratch allocation"));
   e = cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(h->d_partials, 0, sizeof(double) * slot_doubles(h) * psm::PSM_SLOTS, h->stream);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "scratch initialisation"));
   // the TMA-staged kernel where the shape allows it
   if (tma_shape(h, h->tma_tiling, h->tma_tiling_odd)) {

@@ -6,7 +6,7 @@
 //             field onto eps (Sec. 3), moments, B (Eq. 5/6), u_s = omega x r + v,
 //             Omega^F (Eq. 2 / TRT), Omega^S (Eq. 7/8/9), PSM blend (Eq. 4),
 //             streamed store (Eq. 1), force/torque (Eq. 10/11) reduced in FP64
-//             with a deterministic order (per-warp, per-block, last-block sum).
+//             with a deterministic order (per-warp, per-block, k_reduce_slots).
 //   k_import  write a natural state (or a uniform equilibrium) in a layout
 //   k_export  read a state in its layout and write it natural, unshifted, FP64
 //   k_macro   rho and u per cell (FP64)
@@ -2304,7 +2304,9 @@ static __global__ void __launch_bounds__(PSM_THREADS)
   grid_wait_previous();
   const double* s = slots + blockIdx.x * slot;
   double* o = out + ((first + dir * (long long)blockIdx.x) % cap) * row;
-  sum_partials<PSM_THREADS>(s + 1, (int)s[0], ncomp, o);
+  // a step kernel that refused its launch wrote no slot: whatever is there, stay inside it
+  const double most = (double)((slot - 1) / ncomp), G = s[0];
+  sum_partials<PSM_THREADS>(s + 1, G >= 0.0 && G <= most ? (int)G : 0, ncomp, o);
   if (free_mask == 0u) return;
   __syncthreads();
   const int b = threadIdx.x >> 5;
