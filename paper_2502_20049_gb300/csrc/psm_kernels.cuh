@@ -2034,20 +2034,24 @@ static __device__ __noinline__ double add_tail(double x, int n) { return __fma_r
 // power of two (exactly) so that the largest lies in [1, 2), and each is cut
 // into three integers, multiples of 2^-21, 2^-44 and 2^-67, by adding 1.5 times
 // the power of two whose last place that is (the sum's bits then count from the
-// constant's): no value loses a bit above 2^-68 of the largest, and integer
-// sums are exact, so drho and j are their exact values rounded once (FP64 sums
-// round after every term at 2^-53).  u = j / rho: a reciprocal from
-// rcp.approx with one Newton step, then the quotient corrected by its own
-// remainder, rounded as the division is but for ties in the 2^-27 tail.
-// false (nothing written) for populations or densities outside the range the
-// cuts are made for (also infinities and NaN): macro64 decides those.
+// constant's).  Integer sums are exact: drho and j are their exact values,
+// rounded once, or twice where the third cut is not empty (FP64 sums round
+// after every term at 2^-53).  u = j / rho: a reciprocal from rcp.approx with
+// one Newton step, then the quotient corrected by its own remainder
+// (Markstein's method), rounded as the division is but for ties in the 2^-27
+// tail.
+// false (nothing written) for cells that the cuts are not made for, which
+// macro64 decides: a bit below 2^-67 of the largest population (its FP64 sum
+// may consist of such values alone), a largest population of 2 or more (a
+// scale below 1 could push small ones out of range) or below 2^-97, densities
+// outside the range, infinities and NaN.
 template <int Q>
 __device__ __forceinline__ bool macro_int(const float (&f)[Q], double rho0, double& rho, double (&u)[3]) {
   unsigned big = 0u;
 #pragma unroll
   for (int i = 0; i < Q; ++i) big = max(big, __float_as_uint(f[i]) & 0x7fffffffu);
   const int E = (int)(big >> 23);
-  if (E < 30 || E > 250) {
+  if (E < 30 || E > 127) {
     if (big != 0u) return false;
     rho = rho0;
     u[0] = u[1] = u[2] = 0.0;
@@ -2056,12 +2060,14 @@ __device__ __forceinline__ bool macro_int(const float (&f)[Q], double rho0, doub
   const float scale = __uint_as_float((unsigned)(254 - E) << 23);  // 2^(127 - E)
   const float M1 = 6.0f, M2 = 7.152557373046875e-07f, M3 = 8.526512829121202e-14f;  // 1.5 2^2, 2^-21, 2^-44
   int n1[4] = {0, 0, 0, 0}, n2[4] = {0, 0, 0, 0}, n3[4] = {0, 0, 0, 0};  // sums: 1, c_x, c_y, c_z
+  unsigned rest = 0u;  // what the third cut leaves, or-ed
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const float g = __fmul_rn(f[i], scale);
     const float t1 = __fadd_rn(g, M1), r1 = __fsub_rn(g, __fsub_rn(t1, M1));
     const float t2 = __fadd_rn(r1, M2), r2 = __fsub_rn(r1, __fsub_rn(t2, M2));
     const float t3 = __fadd_rn(r2, M3);
+    rest |= __float_as_uint(__fsub_rn(r2, __fsub_rn(t3, M3)));
     const int a = __float_as_int(t1), b = __float_as_int(t2), c = __float_as_int(t3);
     const int s[4] = {1, lat_cx(i), lat_cy(i), lat_cz(i)};
 #pragma unroll
@@ -2070,6 +2076,7 @@ __device__ __forceinline__ bool macro_int(const float (&f)[Q], double rho0, doub
       if (s[k] < 0) n1[k] = (int)((unsigned)n1[k] - (unsigned)a), n2[k] = (int)((unsigned)n2[k] - (unsigned)b), n3[k] = (int)((unsigned)n3[k] - (unsigned)c);
     }
   }
+  if ((rest & 0x7fffffffu) != 0u) return false;
   // the constants' own bits cancel in the sums over c (as many +1 as -1)
   n1[0] = (int)((unsigned)n1[0] - (unsigned)Q * __float_as_uint(M1));
   n2[0] = (int)((unsigned)n2[0] - (unsigned)Q * __float_as_uint(M2));

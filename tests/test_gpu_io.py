@@ -164,3 +164,60 @@ def test_arrays_that_overlap_the_state_are_staged():
     assert np.array_equal(buf.cpu().numpy(), want)
     sol.set_state(buf)
     assert np.array_equal(sol.get_state(), want)
+
+
+def macro_cells(storage):
+    """Populations [19, cells] whose momentum lies far below the largest population of the cell, and per
+    cell and axis whether its FP64 sum is exact (at most one value that does not cancel with the next)."""
+    Q = 19
+    dt = {"fp32": np.float32, "bf16": np.float32}[storage]
+    f, exact = [], []
+    for e in range(-110, -30, 3):       # f_0 alone above values of 2^e; opposite pairs are (1, 2), (3, 4), (5, 6)
+        m = 1.2345678 if storage == "fp32" else 1.2421875
+        a = np.zeros(Q, dt)
+        a[0], a[3] = 0.01, m * 2.0 ** e
+        f.append(a)
+        exact.append((True, True, True))
+        a = a.copy()
+        a[1] = a[2] = 0.0078125          # cancels exactly on x
+        a[5] = -m * 2.0 ** (e - 7)
+        f.append(a)
+        exact.append((True, True, True))
+        a = a.copy()
+        a[7:15] = (1 + np.arange(8) / 8) * 2.0 ** (e + np.arange(8) % 5) * (-1.0) ** np.arange(8)
+        f.append(a)
+        exact.append((False, False, False))
+    return np.array(f).T.copy(), exact
+
+
+@pytest.mark.parametrize("storage", ["fp32", "bf16"])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 9])
+def test_macroscopic_keeps_momentum_far_below_the_largest_population(storage, scale):
+    """A momentum made of populations 2^-110 to 2^-30 of the cell's largest (a rest population, or a pair
+    that cancels): no digit may be lost.  Where the FP64 sum is exact, u is four roundings from exact
+    (density, quotient); elsewhere each of the Q additions may round at the size of the populations that
+    carry momentum on the axis (2 Q eps sum |f_i c_i|)."""
+    import torch
+    from paper_2502_20049_gb300 import psm
+
+    Q = 19
+    f, exact = macro_cells(storage)
+    f = f * np.float32(scale)            # a scale of 2^9 makes the largest population exceed 2
+    n = f.shape[1]
+    buf = torch.from_numpy(f).to(getattr(torch, TORCH_DT[storage])).reshape(Q, 1, 1, n).cuda()
+    sol = solver(storage, Q, (n, 1, 1), bufs=[buf])
+    rho, u = sol.macroscopic()
+    rho, u = rho.reshape(-1), u.reshape(-1, 3)
+    c, _, _ = psm.lattice_velocities(Q)
+    g = buf.cpu().double().numpy().reshape(Q, n)
+    eps = 2.0 ** -53
+    for k in range(n):
+        wr = math.fsum([1.0] + list(g[:, k]))
+        assert abs(rho[k] - wr) <= (2 * abs(wr) + Q * np.abs(g[:, k]).sum()) * eps, k
+        for a in range(3):
+            terms = [g[i, k] * c[i, a] for i in range(Q)]
+            want = math.fsum(terms) / wr
+            tol = 4 * eps * abs(want)
+            if not exact[k][a]:
+                tol += 2 * Q * eps * sum(map(abs, terms)) / wr
+            assert abs(u[k, a] - want) <= tol, (k, a, u[k, a], want)
