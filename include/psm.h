@@ -508,7 +508,8 @@ int psm_check_device_buffer(const void* p, int64_t bytes);
 #define PSM_KERNEL_TMA 2
 int psm_set_kernel_variant(psm_handle h, int variant);
 /* The variant psm_step uses now (PSM_KERNEL_PLAIN or PSM_KERNEL_TMA; under
- * PSM_KERNEL_AUTO: PSM_KERNEL_TMA where the shape allows it). */
+ * PSM_KERNEL_AUTO: PSM_KERNEL_TMA where the shape allows it, but for FP64
+ * grids of at most 256 cells per SM). */
 int psm_kernel_variant(psm_handle h, int* out);
 
 /* Diagnostics (host only, no GPU needed): the shared-memory layout the

@@ -1717,7 +1717,7 @@ int psm_set_kernel_variant(psm_handle h, int variant) {
 
 int psm_kernel_variant(psm_handle h, int* out) {
   if (!valid_handle(h) || !out) return fail(PSM_ERR_ARG, "psm_kernel_variant: NULL argument");
-  *out = (h->tma_ok && h->variant != PSM_KERNEL_PLAIN) ? PSM_KERNEL_TMA : PSM_KERNEL_PLAIN;
+  *out = (h->tma_ok && h->variant != PSM_KERNEL_PLAIN && !fine_grid(h)) ? PSM_KERNEL_TMA : PSM_KERNEL_PLAIN;
   return PSM_OK;
 }
 

@@ -102,3 +102,35 @@ def test_pairs_of_a_varying_flow_equal_plain_bitwise(dims, storage, fluid, Q, st
         s.init_equilibrium_field(rho, u)
         s.step(c.steps)
     assert np.array_equal(a.get_state(), b.get_state())
+
+
+@pytest.mark.parametrize("dims,auto", [((32, 32, 32), "plain"), ((64, 64, 64), "tma"), ((37, 23, 19), "plain")])
+def test_variant_names_the_kernel_that_runs_fp64(dims, auto):
+    """FP64 grids of at most 256 cells per SM take plain loads under AUTO, larger
+    ones of a TMA shape the TMA-staged kernel; forced variants are what was forced."""
+    from paper_2502_20049_gb300 import psm
+
+    s = psm.Solver(psm.SolverConfig(*dims, storage="fp64"))
+    assert s.kernel_variant == auto
+    s.set_kernel_variant("plain")
+    assert s.kernel_variant == "plain"
+    if dims[0] != 37:
+        s.set_kernel_variant("tma")
+        assert s.kernel_variant == "tma"
+    s.set_kernel_variant("auto")
+    assert s.kernel_variant == auto
+
+
+@pytest.mark.parametrize("streaming", ["aa", "twogrid"])
+def test_small_fp64_grid_with_the_tma_kernel_matches_the_oracle(streaming):
+    """The TMA-staged FP64 kernel on a grid where AUTO takes plain loads; 17 steps: more than one sum of loads."""
+    from paper_2502_20049_gb300 import psm
+
+    c = case((64, 16, 12), "fp64", streaming, nb=3, steps=17)
+    s = psm.Solver.from_case(c)
+    s.set_kernel_variant("tma")
+    s.step(c.steps)
+    g = dict(f=s.get_state(), ft=np.stack([s.force_torque(b) for b in range(3)], axis=1))
+    o = run_oracle(c)
+    assert np.abs(g["f"] - o["f"][perm_lib_to_oracle(19)]).max() <= 1e-13
+    assert ft_err(g, o) <= 1e-10
