@@ -87,3 +87,26 @@ def test_bad_meshes_are_refused_on_the_gpu():
     vv, tt = W.merge_meshes(a, b)
     uniq, inv = np.unique(vv, axis=0, return_inverse=True)
     assert psm.voxelize_mesh(uniq.astype(np.float32), inv.reshape(-1)[tt].astype(np.int32), 2).subcells().sum() > 0
+
+
+def test_loose_triangles_are_refused_at_once_whatever_their_number():
+    """Triangles without a common edge have three distinct edges each; 349,525
+    of them are one edge short of 2^20, a power of two that a table of the edges
+    must not be filled to (262,144 leave a quarter of it free)."""
+    import time
+
+    from paper_2502_20049_gb300 import psm
+
+    def refuse(nt):
+        v = np.random.default_rng(5).random((3 * nt, 3), dtype=np.float32)
+        t = np.arange(3 * nt, dtype=np.int32).reshape(-1, 3)
+        best = np.inf
+        for _ in range(3):
+            t0 = time.perf_counter()
+            with pytest.raises(psm.PSMError, match="not closed"):
+                psm.voxelize_mesh(v, t, 1)
+            best = min(best, time.perf_counter() - t0)
+        return best
+
+    few, many = refuse(262144), refuse(349525)
+    assert many <= 10 * few, (few, many)
