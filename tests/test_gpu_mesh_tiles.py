@@ -110,3 +110,18 @@ def test_loose_triangles_are_refused_at_once_whatever_their_number():
 
     few, many = refuse(262144), refuse(349525)
     assert many <= 10 * few, (few, many)
+
+
+@pytest.mark.parametrize("side", [1446, 1450])
+def test_grids_of_many_tiles(side):
+    """A thin box on either side of 2^17 tiles (362^2 and 363^2; more take their
+    counts from an allocation of their own): faces on cell faces, so whole cells
+    are inside or outside."""
+    from paper_2502_20049_gb300 import psm
+
+    v, t = W.box_mesh((0, 0, 0), (1, side, side))
+    g = psm.voxelize_mesh(v, t, 2)
+    w = g.words().reshape(side + 2, side + 2, 3)
+    want = np.zeros_like(w)
+    want[1:-1, 1:-1, 1] = np.iinfo(w.dtype).max
+    assert np.array_equal(w, want)
