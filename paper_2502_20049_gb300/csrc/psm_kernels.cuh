@@ -440,7 +440,8 @@ __device__ __forceinline__ void store_slot(double* slot, const double* blk, int 
 //     step, two-grid 289.6 -> 242.1 (pairs alone: 277.5 and 274.4).
 template <class S, int FL, int MODE>
 __host__ __device__ constexpr bool tile_pairs() {
-  return sizeof(S) == 2 && MODE >= 0 && (FL == 2 || MODE == MODE_AA_ODD);
+  // (tensor stores write one cell per thread)
+  return sizeof(S) == 2 && MODE >= 0 && (FL == 2 || MODE == MODE_AA_ODD) && !(PSM_TMA_STORE && MODE == MODE_AA_EVEN);
 }
 template <class S, int Q, int FL = 0, int MODE = -1>
 __host__ __device__ constexpr int step_min_blocks() {
