@@ -1414,7 +1414,19 @@ struct TmaLayout {
   static constexpr int clamp_st(int n) { return n < 2 ? 2 : (n > PSM_TMA_MAX_STAGES ? PSM_TMA_MAX_STAGES : n); }
   // output boxes per warp: PSM_TMA_OUT_BUFS where that leaves at least 3 input stages, else 1
   static constexpr int NOUT = (PSM_TMA_OUT_BUFS > 1 && (BUDGET0 - PSM_TMA_OUT_BUFS * OUT) / STAGE >= 3) ? PSM_TMA_OUT_BUFS : 1;
-  static constexpr int NST = clamp_st((BUDGET0 - NOUT * OUT) / STAGE);
+  // a multiple of the groups of warps that take alternate tiles (tile_pairs): a
+  // stage then always belongs to one group, whose own waits order its refills
+  static constexpr int GROUPS = tile_pairs<S, FL, MODE>() ? 2 : 1;
+  static constexpr int NST = clamp_st((BUDGET0 - NOUT * OUT) / STAGE) / GROUPS * GROUPS;
+  // refill lag in tiles: a stage is refilled LAG tiles after it was read, so the
+  // refilling warp seldom waits for the slowest warp; NST - LAG tiles stay ahead
+  // (a multiple of the groups too: a warp refills stages that its own group has read)
+#ifdef PSM_TMA_REFILL_LAG
+  static constexpr int LAG0 = PSM_TMA_REFILL_LAG < NST - 1 ? PSM_TMA_REFILL_LAG : NST - 2;
+#else
+  static constexpr int LAG0 = NST >= 5 ? 2 : (NST >= 3 ? 1 : 0);
+#endif
+  static constexpr int LAG = LAG0 / GROUPS * GROUPS;
   // + 128 B of barriers, + 128 B of alignment slack
   static constexpr int SMEM = 256 + NST * STAGE + NOUT * OUT;
 };
@@ -1443,13 +1455,7 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
   using L = TmaLayout<S, Q, MODE, FL>;
   constexpr int NST = L::NST;
   constexpr int NOUT = L::NOUT;
-  // refill lag in tiles: a stage is refilled LAG tiles after it was read, so the
-  // refilling warp seldom waits for the slowest warp; NST - LAG tiles stay ahead
-#ifdef PSM_TMA_REFILL_LAG
-  constexpr int LAG = PSM_TMA_REFILL_LAG < NST - 1 ? PSM_TMA_REFILL_LAG : NST - 2;
-#else
-  constexpr int LAG = NST >= 5 ? 2 : (NST >= 3 ? 1 : 0);
-#endif
+  constexpr int LAG = L::LAG;
   constexpr int EP = L::EP;
   __shared__ double s_ft[PSM_THREADS / 32][PSM_MAX_BODIES * 6];
   __shared__ int s_abort;
@@ -1469,8 +1475,8 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
   // tile_pairs: the even warps take the block's even tiles and the odd warps its
   // odd ones, two x-neighbour cells per thread; otherwise all warps share each tile
   constexpr bool PAIRS = tile_pairs<S, FL, MODE>();
-  constexpr int GROUPS = PAIRS ? 2 : 1;
-  static_assert(GROUPS == 1 || LAG % GROUPS == 0, "a warp refills stages that its own group has read");
+  constexpr int GROUPS = L::GROUPS;
+  static_assert(NST >= GROUPS && NST % GROUPS == 0 && LAG % GROUPS == 0, "a warp refills stages that its own group has read");
   const int nb = p.nft;  // bodies whose loads are wanted
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int k = lane; k < PSM_MAX_BODIES * 6; k += 32) s_ft[warp][k] = 0.0;

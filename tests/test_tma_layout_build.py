@@ -4,6 +4,8 @@ here, not run): what its pipeline and its stores take for granted."""
 import os
 import subprocess
 
+import pytest
+
 from paper_2502_20049_gb300 import build as B
 
 
@@ -29,3 +31,16 @@ def test_tensor_stores_come_with_one_cell_per_thread(tmp_path):
         f"static_assert(!TmaLayout<{s}, {q}, {m}, {f}>::STORE_TMA || (!tile_pairs<{s}, {f}, {m}>() && "
         f"TmaLayout<{s}, {q}, {m}, {f}>::CPT == 1));\n" for s, q, m, f in KINDS)
     assert compiles(tmp_path, ["PSM_TMA_STORE=1", "PSM_TMA_CPT16=1"], asserts) == ""
+
+
+@pytest.mark.parametrize("defines", [[], ["PSM_TMA_MAX_STAGES=2"], ["PSM_TMA_MAX_STAGES=4"], ["PSM_TMA_MAX_STAGES=5"],
+                                     ["PSM_TMA_MAX_STAGES=7", "PSM_TMA_REFILL_LAG=1"], ["PSM_TMA_REFILL_LAG=3"]])
+def test_a_stage_belongs_to_one_group_of_warps(tmp_path, defines):
+    """Where two groups of warps take alternate tiles, tiles k and k + stages
+    share a stage and must fall to one group, and so must a tile and the one at
+    whose reading its stage is refilled: both counts even, whatever the limits."""
+    asserts = "template <class L, bool P> constexpr bool ok() {\n" \
+              "  return L::NST >= 2 && L::LAG >= 0 && L::LAG < L::NST && (!P || (L::NST % 2 == 0 && L::LAG % 2 == 0));\n}\n"
+    asserts += "".join(f"static_assert(ok<TmaLayout<{s}, {q}, {m}, {f}>, tile_pairs<{s}, {f}, {m}>()>());\n"
+                       for s, q, m, f in KINDS)
+    assert compiles(tmp_path, defines, asserts) == ""
