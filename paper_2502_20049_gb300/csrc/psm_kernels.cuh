@@ -1774,11 +1774,9 @@ __global__ void __launch_bounds__(PSM_THREADS, step_min_blocks<S, Q, FL, MODE>()
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned io_plane(const IoParams& p) { return (unsigned)p.g.nx * (unsigned)p.g.ny; }
 
-// The conversion instructions, for the values the bit operations leave out
-// (out of line: inline, the compiler would run them for every value and select).
+// The conversion instruction, for the values the bit operations leave out
+// (out of line: inline, the compiler would run it for every value and select).
 static __device__ __noinline__ double widen_rare(float f) { return (double)f; }
-template <class S>
-static __device__ __noinline__ S narrow_rare(double d) { return Store<S>::from_double(d); }
 
 // double(f): sign, exponent and mantissa moved to their places
 __device__ __forceinline__ double widen(float f) {
@@ -1799,10 +1797,7 @@ __device__ __forceinline__ S narrow(double d) {
   const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), m = hi & 0x7fffffffu;
   // exponents of [2^-126, 2^127): below the smallest normal float, or so large
   // that rounding could overflow, the conversion instruction decides
-  if (m - 0x38100000u >= 0x0fd00000u) {
-    if ((m | lo) == 0u) return Store<S>::from_double(d);
-    return Store<S>::from_double(d);
-  }
+  if (m - 0x38100000u >= 0x0fd00000u) return Store<S>::from_double(d);
   const unsigned top = ((m - 0x38000000u) << 3) | (lo >> 29);
   if constexpr (sizeof(S) == 4) {
     const unsigned rest = lo << 3;  // the 29 discarded bits, left-justified
