@@ -1121,7 +1121,10 @@ int psm_get_cells(psm_handle h, const int64_t* cells, int64_t n, double* f) {
 int psm_get_macroscopic(psm_handle h, double* rho, double* u) {
   if (!valid_handle(h) || !rho || !u) return fail(PSM_ERR_ARG, "psm_get_macroscopic: NULL argument");
   const size_t cells8 = sizeof(double) * (size_t)h->g.ncell;
-  if (direct_array(h, rho, cells8, sizeof(double)) && direct_array(h, u, 3 * cells8, sizeof(double))) {
+  // (arrays that overlap are staged: chunk by chunk rho, then u)
+  const uintptr_t ra = reinterpret_cast<uintptr_t>(rho), ua = reinterpret_cast<uintptr_t>(u);
+  if ((ra + cells8 <= ua || ua + 3 * cells8 <= ra) && direct_array(h, rho, cells8, sizeof(double)) &&
+      direct_array(h, u, 3 * cells8, sizeof(double))) {
     IoParams p;
     io_base(h, p);
     p.z_end = (int)h->grid.nz;

@@ -221,3 +221,20 @@ def test_macroscopic_keeps_momentum_far_below_the_largest_population(storage, sc
             if not exact[k][a]:
                 tol += 2 * Q * eps * sum(map(abs, terms)) / wr
             assert abs(u[k, a] - want) <= tol, (k, a, u[k, a], want)
+
+
+@pytest.mark.parametrize("at", [0, 100, 2200])
+def test_density_and_velocity_into_overlapping_arrays(at):
+    """A caller that wants the velocity alone may let the density array lie
+    anywhere in the velocity's: the velocity is what stays."""
+    import torch
+
+    dims = (37, 5, 7)
+    n = int(np.prod(dims))
+    sol = solver("fp32", dims=dims)
+    z, y, x = np.meshgrid(np.arange(7), np.arange(5), np.arange(37), indexing="ij")
+    sol.init_equilibrium_field(1.0 + 0.01 * np.sin(0.3 * x + y), 0.02 * np.stack([np.sin(0.5 * x), np.cos(y + z), 0.1 * z], -1))
+    _, want = sol.macroscopic()
+    u = torch.empty((7, 5, 37, 3), dtype=torch.float64, device="cuda")
+    sol.macroscopic(u.view(-1)[at:at + n], u)
+    assert np.array_equal(u.cpu().numpy(), want)
