@@ -238,3 +238,38 @@ def test_density_and_velocity_into_overlapping_arrays(at):
     u = torch.empty((7, 5, 37, 3), dtype=torch.float64, device="cuda")
     sol.macroscopic(u.view(-1)[at:at + n], u)
     assert np.array_equal(u.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("kind", ["managed", "pinned"])
+def test_arrays_in_managed_and_pinned_memory(kind):
+    """Managed memory takes the direct kernels, pinned host memory the staging
+    chunk: the bits of an array on the device."""
+    import ctypes
+
+    import torch
+
+    dims = (37, 5, 7)
+    sol = solver("fp32", dims=dims)
+    sol.init_equilibrium(1.02, (0.01, -0.02, 0.03))
+    want = sol.get_state(torch.empty(sol.shape, dtype=torch.float64, device="cuda")).cpu().numpy()
+    n = want.size
+    if kind == "pinned":
+        a = torch.empty(sol.shape, dtype=torch.float64).pin_memory()
+        sol.get_state(a)
+        got = a.numpy()
+        sol.init_equilibrium(1.0, (0.0, 0.0, 0.0))
+        sol.set_state(a)
+    else:
+        from paper_2502_20049_gb300 import psm
+
+        rt = ctypes.CDLL("/usr/local/cuda/lib64/libcudart.so")
+        p = ctypes.c_void_p()
+        assert rt.cudaMallocManaged(ctypes.byref(p), ctypes.c_size_t(8 * n), ctypes.c_uint(1)) == 0
+        psm.check(psm.lib().psm_get_state(sol._h, p))
+        got = np.ctypeslib.as_array(ctypes.cast(p, ctypes.POINTER(ctypes.c_double)), shape=(n,)).reshape(want.shape).copy()
+        sol.init_equilibrium(1.0, (0.0, 0.0, 0.0))
+        psm.check(psm.lib().psm_set_state(sol._h, p))
+        sol.synchronize()
+        assert rt.cudaFree(p) == 0
+    assert np.array_equal(got, want)
+    assert np.array_equal(sol.get_state(), want)

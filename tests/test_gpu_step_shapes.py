@@ -134,3 +134,42 @@ def test_small_fp64_grid_with_the_tma_kernel_matches_the_oracle(streaming):
     o = run_oracle(c)
     assert np.abs(g["f"] - o["f"][perm_lib_to_oracle(19)]).max() <= 1e-13
     assert ft_err(g, o) <= 1e-10
+
+
+@pytest.mark.parametrize("storage,dims", [("fp32", (64, 16, 12)), ("fp16", (256, 8, 12)), ("fp64", (33, 12, 9))])
+def test_steps_between_a_callers_kernels_on_its_stream(storage, dims):
+    """psm_step on a side stream, its launches overlapped, between kernels of the
+    caller on the same stream that write the PDF buffer before and read it after
+    each call, without a synchronisation: as on the default stream with one."""
+    import torch
+    from paper_2502_20049_gb300 import psm
+
+    c = case(dims, storage, "aa", nb=2)
+    cfg = psm.SolverConfig(*dims, storage=storage, fluid="trt", tau=0.65, u_in=(0.02, -0.01, 0.03))
+    dt = {"fp64": torch.float64, "fp32": torch.float32, "fp16": torch.float16}[storage]
+    fields = [(psm.voxelize(b.kind, b.params, b.s), b) for b in c.bodies]
+    start = (0.01 * torch.rand((19,) + dims[::-1], generator=torch.Generator().manual_seed(3))).to(dt).cuda()
+
+    def run(stream, wait):
+        with torch.cuda.stream(stream):
+            f = torch.zeros_like(start)
+            sol = psm.Solver(cfg, buffers=[f], keep=True)
+            for k, (g, b) in enumerate(fields):
+                sol.set_geometry(k, g, np.array(b.Q0), b.R0, b.omega, b.v)
+            seen = []
+            for n in (1, 2, 3, 18):
+                f.copy_(start + f * 0.5)
+                if wait:
+                    torch.cuda.synchronize()
+                sol.step(n)
+                seen.append(f.clone())
+                if wait:
+                    torch.cuda.synchronize()
+            return [x.cpu() for x in seen], [sol.force_torque(k) for k in range(2)]
+
+    a, fa = run(torch.cuda.Stream(), False)
+    b, fb = run(torch.cuda.default_stream(), True)
+    for x, y in zip(a, b):
+        assert torch.equal(x, y)
+    for x, y in zip(fa, fb):
+        assert np.array_equal(x, y)
