@@ -518,7 +518,8 @@ int psm_kernel_variant(psm_handle h, int* out);
  *   out[0] dynamic shared memory per block (bytes), out[1] pipeline stages,
  *   out[2] resident blocks per SM it is sized for, out[3] cells per thread.
  * The stages fill 228 KB per SM over out[2] blocks, less 1 KB reserved and
- * 6 KB of static shared memory per block.  PSM_ERR_ARG for an unknown value,
+ * 6 KB of static shared memory per block (an even number where two groups of
+ * warps take alternate tiles).  PSM_ERR_ARG for an unknown value,
  * PSM_ERR_UNSUPPORTED for the cumulant operator on D3Q27. */
 int psm_tma_layout(int storage, int stencil, int mode, int fluid, int* out);
 

@@ -616,14 +616,18 @@ bool encode_maps(const psm_solver* h, void* buf, BufMaps& m, const psm::Tiling& 
   return r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS && r3 == CUDA_SUCCESS;
 }
 
-// FP64 storage under PSM_KERNEL_AUTO on a grid of fewer 256-cell blocks than the
-// GPU has SMs: the plain kernel with blocks of 64 cells.  FP64 arithmetic bounds
-// the step (an SM issues one FP64 warp instruction in about 16 clocks), so the
-// cells of a body, the slow ones above all, are spread over four times as many
-// blocks: 32^3 with a sphere 33 us a step, 43 us in blocks of 256 (plain or
-// TMA).  Below FP64 the same split only adds blocks to the load reduction (32^3
-// FP32 12.3 us in blocks of 256, 14.3 us in blocks of 64), and on larger grids
-// every SM has several blocks either way.
+// FP64 storage under PSM_KERNEL_AUTO on a grid of at most as many 256-cell
+// blocks as the GPU has SMs: the plain kernel with blocks of 64 cells.  FP64
+// arithmetic bounds the step (an SM issues one FP64 warp instruction in about 16
+// clocks), so the cells of a body, the slow ones above all, are spread over four
+// times as many blocks.  us a step, D3Q19 BGK, 64-thread blocks / 256 / TMA:
+// 32^3 with a sphere 24.9 / 35.6 / 36.2, without 11.8 / 12.2 / 12.5; 64x16x32
+// with a sphere 25.2 / 40.2 / 40.5; 256x8x16 25.7 / 28.9 / 24.9; the worst found,
+// 33x31x36 D3Q27, 62 / 51.  Below FP64 the same split only adds blocks to the
+// load reduction (32^3 FP32 12.3 us in blocks of 256, 14.3 us in blocks of 64).
+// The line is where every SM still has one block of 256 at most; forced beyond it
+// the small blocks gain on rows of up to 64 cells (64x64x32 with a sphere
+// 52 / 68 / 67, 64^3 101 / 128 / 128) and lose up to 6 % on rows of 256.
 bool fine_grid(const psm_solver* h) {
   const long long sms = h->max_blocks / (2048 / psm::PSM_THREADS);
   return h->lat.storage == PSM_FP64 && h->variant == PSM_KERNEL_AUTO && h->g.ncell <= sms * psm::PSM_THREADS;

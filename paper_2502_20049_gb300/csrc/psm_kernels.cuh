@@ -430,13 +430,15 @@ __device__ __forceinline__ void store_slot(double* slot, const double* blk, int 
 // storage): a tile is four warps' work, and the block's two groups of warps take
 // alternate tiles.  These steps are bound by instruction issue, and a pair shares
 // shared-memory accesses, stores, addresses and the tile's bookkeeping.
-//   AA odd, BGK/TRT: 545 -> 343 warp instructions per 32 cells (D3Q19).  Two-row
-//     tiles for the pairs halved the pipeline's depth; one-row tiles keep it.
+//   AA odd, BGK/TRT: 539 -> 403 warp instructions per 32 cells (D3Q19, 256x256x240
+//     with two rotors), 644 -> 527 (D3Q27, 256x256x320).  Two-row tiles for the pairs
+//     halved the pipeline's depth; one-row tiles keep it.
 //     1024x1024x960 D3Q19 FP16 14.11 -> 13.67 ms per AA step (even and odd
 //     averaged), 512x512x640 D3Q27 3.456 -> 3.348.
 //   Cumulant, every mode: the additions and multiply-adds of its arithmetic
-//     (about 240 of 449 instructions per 32 cells) are packed FP32 instructions
-//     as well; 128 registers without spills.  256^3 FP16 AA 296.8 -> 245.6 us a
+//     are packed FP32 instructions as well (256^3: AA even 449 -> 302 warp
+//     instructions per 32 cells, AA odd 530 -> 402, two-grid 491 -> 343); 128
+//     registers without spills.  256^3 FP16 AA 296.8 -> 245.6 us a
 //     step, two-grid 289.6 -> 242.1 (pairs alone: 277.5 and 274.4).
 template <class S, int FL, int MODE>
 __host__ __device__ constexpr bool tile_pairs() {
@@ -1194,8 +1196,9 @@ __device__ __forceinline__ void fluid_collide2(const StepParams& p, F2 (&f)[Q]) 
 // cell box, lies in no plane next to a ghost plane and no eps perturbation is
 // set (tile_general, for its 32 cells).  The force/torque partials are those of
 // 32 x-neighbours whatever the block size; where the TMA kernel applies, blocks
-// of 256 hold its tiles' cells in the same order, so that the sums agree bit for
-// bit.  96x96x120 D3Q27 FP32 with two rotors: 67 us a step in whole-row tiles,
+// of 256 hold its tiles' cells in the same order, so that in FP32 and FP64
+// storage the sums agree bit for bit (in 16-bit storage its warps hold other
+// cells).  96x96x120 D3Q27 FP32 with two rotors: 67 us a step in whole-row tiles,
 // 58 us in units; 203x117x151 FP16 88 and 85 us.
 // ---------------------------------------------------------------------------
 template <class S, int Q, int MODE, int FL, int NT>
