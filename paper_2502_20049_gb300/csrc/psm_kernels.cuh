@@ -2039,8 +2039,8 @@ static __device__ __noinline__ double add_tail(double x, int n) { return __fma_r
 // power of two (exactly) so that the largest lies in [1, 2), and each is cut
 // into three integers, multiples of 2^-21, 2^-44 and 2^-67, by adding 1.5 times
 // the power of two whose last place that is (the sum's bits then count from the
-// constant's).  Integer sums are exact: drho and j are their exact values,
-// rounded once, or twice where the third cut is not empty (FP64 sums round
+// constant's).  Integer sums are exact, and so are drho and j, but for one rounding
+// where the third cut is not empty; rho0 + drho is rounded once (FP64 sums round
 // after every term at 2^-53).  u = j / rho: a reciprocal from rcp.approx with
 // one Newton step, then the quotient corrected by its own remainder
 // (Markstein's method), rounded as the division is but for ties in the 2^-27
