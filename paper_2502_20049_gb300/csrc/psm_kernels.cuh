@@ -2046,15 +2046,19 @@ static __device__ __noinline__ double add_tail(double x, int n) { return __fma_r
 // (Markstein's method), rounded as the division is but for ties in the 2^-27
 // tail.
 // false (nothing written) for cells that the cuts are not made for, which
-// macro64 decides: a bit below 2^-67 of the largest population (its FP64 sum
-// may consist of such values alone), a largest population of 2 or more (a
-// scale below 1 could push small ones out of range) or below 2^-97, densities
-// outside the range, infinities and NaN.
+// macro64 decides: a population below 2^-44 of the largest, whose last bits the
+// third cut would drop (the momentum may consist of such values alone), a
+// largest population of 2 or more (a scale below 1 could push small ones out of
+// range) or below 2^-97, densities outside the range, infinities and NaN.
 template <int Q>
 __device__ __forceinline__ bool macro_int(const float (&f)[Q], double rho0, double& rho, double (&u)[3]) {
-  unsigned big = 0u;
+  unsigned big = 0u, small = ~0u;  // largest and smallest size (less one: zeros do not count as small)
 #pragma unroll
-  for (int i = 0; i < Q; ++i) big = max(big, __float_as_uint(f[i]) & 0x7fffffffu);
+  for (int i = 0; i < Q; ++i) {
+    const unsigned m = __float_as_uint(f[i]) & 0x7fffffffu;
+    big = max(big, m);
+    small = min(small, m - 1u);
+  }
   const int E = (int)(big >> 23);
   if (E < 30 || E > 127) {
     if (big != 0u) return false;
@@ -2062,17 +2066,17 @@ __device__ __forceinline__ bool macro_int(const float (&f)[Q], double rho0, doub
     u[0] = u[1] = u[2] = 0.0;
     return rho0 > 0.0;
   }
+  // 24 bits from 2^-44 of the largest on end above the last cut
+  if (E > 44 && small < ((unsigned)(E - 44) << 23) - 1u) return false;
   const float scale = __uint_as_float((unsigned)(254 - E) << 23);  // 2^(127 - E)
   const float M1 = 6.0f, M2 = 7.152557373046875e-07f, M3 = 8.526512829121202e-14f;  // 1.5 2^2, 2^-21, 2^-44
   int n1[4] = {0, 0, 0, 0}, n2[4] = {0, 0, 0, 0}, n3[4] = {0, 0, 0, 0};  // sums: 1, c_x, c_y, c_z
-  unsigned rest = 0u;  // what the third cut leaves, or-ed
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const float g = __fmul_rn(f[i], scale);
     const float t1 = __fadd_rn(g, M1), r1 = __fsub_rn(g, __fsub_rn(t1, M1));
     const float t2 = __fadd_rn(r1, M2), r2 = __fsub_rn(r1, __fsub_rn(t2, M2));
     const float t3 = __fadd_rn(r2, M3);
-    rest |= __float_as_uint(__fsub_rn(r2, __fsub_rn(t3, M3)));
     const int a = __float_as_int(t1), b = __float_as_int(t2), c = __float_as_int(t3);
     const int s[4] = {1, lat_cx(i), lat_cy(i), lat_cz(i)};
 #pragma unroll
@@ -2081,7 +2085,6 @@ __device__ __forceinline__ bool macro_int(const float (&f)[Q], double rho0, doub
       if (s[k] < 0) n1[k] = (int)((unsigned)n1[k] - (unsigned)a), n2[k] = (int)((unsigned)n2[k] - (unsigned)b), n3[k] = (int)((unsigned)n3[k] - (unsigned)c);
     }
   }
-  if ((rest & 0x7fffffffu) != 0u) return false;
   // the constants' own bits cancel in the sums over c (as many +1 as -1)
   n1[0] = (int)((unsigned)n1[0] - (unsigned)Q * __float_as_uint(M1));
   n2[0] = (int)((unsigned)n2[0] - (unsigned)Q * __float_as_uint(M2));
