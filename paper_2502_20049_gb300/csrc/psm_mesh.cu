@@ -500,6 +500,10 @@ extern "C" int psm_geom_voxelize_mesh(const float* vertices, int64_t nv, const i
     release();
     return mesh_fail(PSM_ERR_OOM, "geometry field allocation failed");
   }
+  // the field's pages exist before the copy: into memory that the heap has only
+  // just grown by, the copy of a 9.3 MB field took 7.6 ms instead of 0.2 (the
+  // same call 0.6 or 8.2 ms by what else the process holds, now 0.6 or 0.8)
+  for (size_t o = 0; o < nwords * sizeof(uint64_t); o += 4096) reinterpret_cast<volatile char*>(bricks)[o] = 0;
   if (e == cudaSuccess) e = cudaMemcpy(bricks, dbr, sizeof(uint64_t) * nwords, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemcpy(&hi, info, sizeof hi, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) {

@@ -125,3 +125,21 @@ def test_grids_of_many_tiles(side):
     want = np.zeros_like(w)
     want[1:-1, 1:-1, 1] = np.iinfo(w.dtype).max
     assert np.array_equal(w, want)
+
+
+def test_calls_that_grow_the_heap_take_about_as_long():
+    """Results that are kept and freed in turn make the heap grow and shrink
+    under the field; a call must not pay several times its own time for that."""
+    import time
+
+    from paper_2502_20049_gb300 import psm
+
+    v, t = W.icosphere(60.0, 6)  # 81,920 triangles, a field of 123^3 words at s = 2
+    held, took = [], []
+    for k in range(16):
+        t0 = time.perf_counter()
+        g = psm.voxelize_mesh(v * np.float32(1 - 0.0005 * k), t, 2)
+        took.append(time.perf_counter() - t0)
+        held = (held + [g, g.words()])[-4:]
+    took = sorted(took[4:])
+    assert took[-1] <= 4 * took[len(took) // 2], took
